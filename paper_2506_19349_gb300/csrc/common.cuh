@@ -39,6 +39,7 @@ struct DevGraph {
   const uint32_t* dcnt0;  // [D] number of vertices with degree dvals[r]
   const uint32_t* dfirst;  // [D] first internal id of degree dvals[r] (decreasing in r: ids run by degree descending)
   const uint2* dhint;      // [ni / 4096 + 1] {rank of the block's last id, rank of its first id} per 4096 ids
+  const uint4* drow;       // [D] {first internal id of degree dvals[r], its row offset, dvals[r], 0}
   uint32_t D;
   const uint32_t* rtow;   // [EIC_RATIO_NUM] maxW(G, i / (RATIO_NUM - 1))
   const uint4* nz;        // [nz_count = ni] {internal id, smallest row weight, row begin, row end}, by (weight, id)
@@ -64,6 +65,14 @@ __device__ __forceinline__ uint32_t degree_rank(const DevGraph& G, uint32_t x) {
       lo = mid + 1;
   }
   return lo;
+}
+
+// Row of internal vertex x as {begin, length}: the rows of one degree follow
+// each other in id order, so both come from the id (three reads of small
+// tables that stay in L1) in place of a random read of row[x], row[x + 1].
+__device__ __forceinline__ uint2 row_of(const DevGraph& G, uint32_t x) {
+  const uint4 t = __ldg(&G.drow[degree_rank(G, x)]);
+  return make_uint2(t.y + (x - t.x) * t.z, t.z);
 }
 
 // ------------------------------------------------------------ warp helpers

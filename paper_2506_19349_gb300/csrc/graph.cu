@@ -308,6 +308,7 @@ void graph_free_arrays(eic_graph* g) {
   cudaFree(g->dcnt0);
   cudaFree(g->dfirst);
   cudaFree(g->dhint);
+  cudaFree(g->drow);
   cudaFree(g->rtow);
   cudaFree(g->nz);
   cudaFree(g->nz_lt);
@@ -524,20 +525,26 @@ int build(eic_graph* g, const uint32_t* src, const uint32_t* dst, const uint32_t
     k_degree_tables<<<grid_for(hlen), kThreads, 0, st>>>(dh, flags, pos, hlen, g->dvals, g->dcnt0, g->drank);
     k_highd0<<<1, 1024, 0, st>>>(g->dcnt0, g->dvals, D, small + 4);
     EIC_CUDA_TRY(cudaGetLastError());
-    // dfirst[r]: the first internal id of degree dvals[r] (ids by degree descending)
+    // dfirst[r]: the first internal id of degree dvals[r] (ids by degree descending); drow[r]: the same with that
+    // id's row offset and the degree
     TRY(galloc(g, &g->dfirst, D));
+    TRY(galloc(g, &g->drow, D));
     if (D) {
       std::vector<uint32_t> cnt(D), first(D), vals(D);
+      std::vector<uint4> rows(D);
       EIC_CUDA_TRY(cudaMemcpyAsync(cnt.data(), g->dcnt0, (uint64_t)D * 4, cudaMemcpyDeviceToHost, st));
       EIC_CUDA_TRY(cudaMemcpyAsync(vals.data(), g->dvals, (uint64_t)D * 4, cudaMemcpyDeviceToHost, st));
       EIC_CUDA_TRY(cudaStreamSynchronize(st));
-      uint64_t acc = 0;
+      uint64_t acc = 0, off = 0;
       for (uint32_t r = D; r-- > 0;) {
         first[r] = (uint32_t)acc;
+        rows[r] = make_uint4((uint32_t)acc, (uint32_t)off, vals[r], 0u);
         acc += cnt[r];
+        off += (uint64_t)cnt[r] * vals[r];
         if (vals[r] > kCursorMin) nlong = (uint32_t)acc;  // ids [0, acc) have degree >= vals[r]
       }
       EIC_CUDA_TRY(cudaMemcpyAsync(g->dfirst, first.data(), (uint64_t)D * 4, cudaMemcpyHostToDevice, st));
+      EIC_CUDA_TRY(cudaMemcpyAsync(g->drow, rows.data(), (uint64_t)D * sizeof(uint4), cudaMemcpyHostToDevice, st));
       EIC_CUDA_TRY(cudaStreamSynchronize(st));
     }
     // dhint[b]: the ranks of ids 4096 b + 4095 and 4096 b (the range a rank search in block b needs)
@@ -611,6 +618,7 @@ int build(eic_graph* g, const uint32_t* src, const uint32_t* dst, const uint32_t
   dg.dcnt0 = g->dcnt0;
   dg.dfirst = g->dfirst;
   dg.dhint = g->dhint;
+  dg.drow = g->drow;
   dg.nlong = nlong;
   dg.D = D;
   dg.rtow = g->rtow;

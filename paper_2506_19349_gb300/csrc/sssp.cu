@@ -127,10 +127,26 @@ struct RoundScr {
 // are staged per warp and written by the warp with one global atomic per
 // kWarpStage entries (no block synchronisation); tasks are staged per block
 // and written at the end of a phase.
+// A fused round has neither tasks nor a staged next frontier: the local
+// queues of its warp groups take their place.
+// Warps that share a local queue: 1, 4, 8 and 16 took 13.3, 7.8, 7.2 and 7.3 ms
+// on a 1531 x 977 grid at gap_shift 4 (long waves: sharing evens out the work)
+// and 123, 117, 119 and 121 ms on a 4096^2 grid (short ones: less to wait for).
+constexpr uint32_t kFuseWarps = 8;
+constexpr uint32_t kFusePop = 8;      // queued vertices a warp takes at a time
+constexpr uint32_t kFuseQueue = 128 * kFuseWarps;  // entries of a local queue (a power of two)
+constexpr uint32_t kFuseGroups = (kMaxWarps + kFuseWarps - 1) / kFuseWarps;
+static_assert(kFuseGroups <= 15, "a group synchronises on named barrier 1 + its index; 0 is the block barrier");
 struct Stage {
   uint32_t tn, tbase;
-  Task tbuf[kStageT];
-  uint32_t wq[kMaxWarps][kWarpStage];
+  union {
+    struct {
+      Task tbuf[kStageT];
+      uint32_t wq[kMaxWarps][kWarpStage];
+    };
+    uint4 fq[kFuseGroups][kFuseQueue];  // {vertex, distance, row begin, degree}
+  };
+  uint32_t fcnt[kFuseGroups][3];  // entries pushed to the local queue, by wave mod 3
   uint32_t wf[kMaxWarps][kWarpStage];
 };
 
@@ -294,6 +310,8 @@ __device__ __forceinline__ uint4 ld_stream4(const uint4* p) {
       : "l"(p), "l"(stream_policy()));
   return v;
 }
+
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // first index in [b, e) of the weight-sorted row with weight >= t
 __device__ __forceinline__ uint32_t lower_bound_w(const uint2* __restrict__ adj, uint32_t b, uint32_t e, int64_t t) {
@@ -972,90 +990,108 @@ __device__ __noinline__ int64_t block_st_exact_call(const KArgs& A, S3Scr& S, in
 // A fused round: the FUSED local iterations of Section 4.1 (bucket fusion),
 // for graphs in which no window is longer than heavy_min (every degree <=
 // heavy_min, so there are no grid tasks), in every round of a step after the
-// first (and its first round too when the step has no pull). Each warp takes
-// up to 32 of the round's frontier vertices (or of the push set, whose windows
-// start at their cursors) and relaxes their windows; every vertex it improves
-// goes into the warp's local queue (shared
-// memory, kWarpStage entries) and is relaxed by the same warp in its next
-// wave, with the distance it has then, until the local queue is empty. The
-// warps advance independently, with no grid barrier between waves: the round
-// replaces the step's remaining rounds. A vertex improved by two warps is
-// relaxed by both, and the smaller distance wins (within a step any order of
-// the relaxations is exact). What a full local queue cannot take goes to the
-// next round's queue through the round's SAP bitmap, as in a plain round.
-// A wave is one chain of dependent loads (the vertex record, its row, the
-// neighbours' distances, the atomicMin) where a plain round adds a grid
-// barrier and the next round's item fetch.
+// first (and its first round too when the step has no pull). The round's
+// frontier vertices (or the push set, whose windows start at their cursors)
+// are dealt evenly to groups of kFuseWarps warps all over the query's blocks.
+// A group relaxes its vertices' windows; every vertex it improves goes into
+// the group's local queue (shared memory, kFuseQueue entries) and is relaxed
+// in a later wave of the group, until the local queue is empty. The groups
+// advance independently, with no grid barrier between waves: the round
+// replaces the step's remaining rounds. A queued vertex that has a smaller
+// distance by the time its wave comes is dropped: whoever lowered it queued it
+// too (within a step any order of the relaxations is exact). What a full
+// local queue cannot take goes to the next round's queue through the round's
+// SAP bitmap, as in a plain round.
+//
+// A wave is bound by its chain of dependent accesses, so the chain is two
+// long: the row's entries, then the atomicMin on the neighbours. Row bounds
+// come from the vertex id (row_of) before the vertex is queued, the check of
+// a queued vertex's distance flies with its row's entries, and a neighbour's
+// row is prefetched into L2 while its atomicMin is under way. Measured against
+// the earlier form (32 items to a warp, one local queue per warp, a chain of
+// row bounds, entries, distance, atomicMin): a round of the 4096^2 grid went
+// from 26.1 to 14.4 us, its query from 168 to 118 ms, and the 1531 x 977 grid
+// at gap_shift 4 from 18.7 to 7.2 ms.
 __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, RoundScr& S, Stage& T,
                             uint32_t nitems, bool round1, const uint32_t* qin, Counters& C) {
   const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
-  const uint32_t gwarp = qblock(A) * (blockDim.x >> 5) + warp;
+  const uint32_t wpb = blockDim.x >> 5, gpb = (wpb + kFuseWarps - 1) / kFuseWarps;
+  const uint32_t grp = warp / kFuseWarps, gw = warp - grp * kFuseWarps;  // the group, the warp's place in it
+  const uint32_t gn = min(kFuseWarps, wpb - grp * kFuseWarps);           // its warps
+  auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(gn * 32) : "memory"); };
   WarpScr& W = S.w[warp];
-  uint32_t* lq = T.wq[warp];  // the local queue: a ring of kWarpStage vertex ids
-  uint32_t lh = 0, lt = 0;    // its head and tail (warp-uniform)
+  uint4* fq = T.fq[grp];  // the local queue: a ring of kFuseQueue entries
+  uint32_t* fcnt = T.fcnt[grp];
   WarpList Fw = {T.wf[warp], 0u, R.first_cnt, R.first_list};
-  const uint32_t i0 = gwarp * 32;
-  // a step's first round (no pull): the warp's first wave is its share of the
-  // push set (and the source, once); later rounds: of the round's queue
+  // the group's share of the items: one block's groups are a grid stride
+  // apart, so that few items still reach every SM
+  const uint32_t per = (nitems + A.nb * gpb - 1) / (A.nb * gpb);
+  uint32_t i0 = min(nitems, (grp * A.nb + qblock(A)) * per);
+  const uint32_t i1 = min(nitems, i0 + per);
   const uint32_t np = round1 ? L.push_end - L.push_beg : 0;
-  uint32_t nseed = round1 && i0 < nitems ? min(32u, nitems - i0) : 0u;
-  if (!round1 && i0 < nitems) {
-    if (i0 + lane < nitems) lq[lane] = ld_list(&qin[i0 + lane]);
-    lt = min(32u, nitems - i0);
-  }
-  __syncwarp();
-  while (nseed || lh != lt) {
-    uint32_t d = EIC_INF, b = 0, len = 0;
-    bool vertex = false;  // a frontier vertex (or the source): its window starts at its row
-    uint32_t u = 0;
-    if (nseed) {
-      const uint32_t i = i0 + lane;
-      if (lane < nseed && i < np) {  // push set entry: settled, lb0 <= dist <= st (Function 1)
+  if (gw == 0 && lane < 3) fcnt[lane] = 0;
+  group_sync();
+  uint32_t lh = 0, lt = 0, wave = 0;  // the ring's head and tail, the wave mod 3 (the same in every thread of the group)
+  while (i0 < i1 || lh != lt) {
+    uint32_t d = EIC_INF, b = 0, len = 0, u = 0, rb = 0, deg = 0;
+    uint32_t now = EIC_INF;  // a queued vertex's distance as its wave begins
+    bool vertex = false;     // a frontier vertex (or the source): its window starts at its row
+    const uint32_t room = kFuseQueue - (lt - lh);
+    if (i0 < i1) {
+      const uint32_t take = min(i1 - i0, 32 * gn), each = (take + gn - 1) / gn;
+      const uint32_t i = i0 + gw * each + lane;
+      const bool mine = lane < each && gw * each + lane < take;
+      i0 += take;
+      if (mine && i < np) {  // push set entry: settled, lb0 <= dist <= st (Function 1)
         const uint32_t idx = L.push_beg + i;
         d = ld_list(&A.sd[idx]);
-        const uint32_t x = ld_list(&A.sid[idx]);
-        const uint2 rr = make_uint2(__ldg(&A.G.row[x]), __ldg(&A.G.row[x + 1]));
-        if ((int64_t)d >= R.lb0 && (int64_t)d <= R.st && !(d > 0 && rr.y - rr.x == 1)) {
+        u = ld_list(&A.sid[idx]);
+        const uint32_t cur = ld_list(&A.scur[idx]);
+        const uint2 rr = row_of(A.G, u);
+        if ((int64_t)d >= R.lb0 && (int64_t)d <= R.st && !(d > 0 && rr.y == 1)) {
           C.frontier += 1;
-          const uint32_t cur = ld_list(&A.scur[idx]);
-          b = cur == kNone ? lower_bound_w(A.G.adj, rr.x, rr.y, R.lb - (int64_t)d)
-                           : gallop_w(A.G.adj, rr.x + cur, rr.y, R.lb - (int64_t)d);
-          const uint32_t e = gallop_w(A.G.adj, b, rr.y, R.ub_eff - (int64_t)d);
-          __stcg(&A.scur[idx], e - rr.x);
-          len = e - b;
+          b = rr.x;
+          len = rr.y;  // a short row: read whole, filtered by the window
+          if (rr.y > kCursorMin) {
+            b = cur == kNone ? lower_bound_w(A.G.adj, rr.x, rr.x + rr.y, R.lb - (int64_t)d)
+                             : gallop_w(A.G.adj, rr.x + cur, rr.x + rr.y, R.lb - (int64_t)d);
+            const uint32_t e = gallop_w(A.G.adj, b, rr.x + rr.y, R.ub_eff - (int64_t)d);
+            __stcg(&A.scur[idx], e - rr.x);
+            len = e - b;
+          }
+          now = d;
         }
-      } else if (lane < nseed) {  // the source, once
-        u = L.s_int;
-        vertex = true;
+      } else if (mine) {  // a frontier vertex, or in a step's first round the source, once
+        u = round1 ? L.s_int : ld_list(&qin[i]);
+        const uint2 rr = row_of(A.G, u);
+        rb = rr.x;
+        deg = rr.y;
+        d = now = __ldcg(&A.dist[u]);
+        vertex = d != EIC_INF && !(d > 0 && deg == 1);  // Paths excludes leaves (Algorithm 1)
       }
-      nseed = 0;
     } else {
-      const uint32_t k = min(32u, lt - lh);
-      if (lane < k) {
-        u = lq[(lh + lane) & (kWarpStage - 1)];
+      const uint32_t take = min(lt - lh, kFusePop * gn), each = (take + gn - 1) / gn;
+      if (lane < each && gw * each + lane < take) {
+        const uint4 q = fq[(lh + gw * each + lane) & (kFuseQueue - 1)];
+        u = q.x;
+        d = q.y;
+        rb = q.z;
+        deg = q.w;
+        now = __ldcg(&A.dist[u]);
         vertex = true;
       }
-      __syncwarp();
-      lh += k;
+      lh += take;
     }
-    if (vertex) {
-      d = __ldcg(&A.dist[u]);
-      const uint32_t rb = __ldg(&A.G.row[u]), re = __ldg(&A.G.row[u + 1]);
+    if (vertex && (int64_t)d < R.ub_eff) {
       // d >= lb: the window is the row's prefix with weight < ub - d; rows are
       // short, so the whole row is read and filtered (a search only for rows
       // that keep a cursor)
-      if (d != EIC_INF && !(d > 0 && re - rb == 1)) {  // Paths excludes leaves (Algorithm 1)
-        C.frontier += 1;
-        const int64_t hi = R.ub_eff - (int64_t)d;
-        if (hi > 0) {
-          b = rb;
-          len = re - rb;
-          if (re - rb > kCursorMin) {
-            const uint32_t e = gallop_w(A.G.adj, rb, re, hi);
-            __stcg(&A.cursor[u], e - rb);
-            len = e - rb;
-          }
-        }
+      b = rb;
+      len = deg;
+      if (deg > kCursorMin) {
+        const uint32_t e = gallop_w(A.G.adj, rb, rb + deg, R.ub_eff - (int64_t)d);
+        __stcg(&A.cursor[u], e - rb);
+        len = e - rb;
       }
     }
     const uint32_t incl = warp_incl_scan(len);
@@ -1064,10 +1100,11 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
     W.excl[lane] = incl - len;
     W.val[lane] = d;
     __syncwarp();
+    uint32_t live = 0;  // lanes whose vertex still has the distance it was queued with
     for (uint32_t g0 = 0; g0 < total; g0 += 32) {
       const uint32_t g = g0 + lane;
-      bool ok = false, first = false;
-      uint32_t v = 0;
+      uint32_t own = 0;
+      uint2 ent = make_uint2(0u, 0u);
       if (g < total) {
         uint32_t lo = 0, hi = 31;
         while (lo < hi) {  // the last lane whose window starts at or before g
@@ -1077,38 +1114,51 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
           else
             hi = mid - 1;
         }
-        const uint2 ent = ld_stream(&A.G.adj[W.beg[lo] + (g - W.excl[lo])]);
-        const uint32_t du = W.val[lo];
-        v = ent.x;
-        if ((int64_t)ent.y < R.ub_eff - (int64_t)du) {
+        own = lo;
+        ent = ld_stream(&A.G.adj[W.beg[lo] + (g - W.excl[lo])]);
+      }
+      if (g0 == 0) {
+        live = __ballot_sync(EIC_FULL_MASK, now == d);
+        C.frontier += vertex && now == d ? 1 : 0;
+      }
+      bool ok = false, first = false;
+      uint32_t nd = 0;
+      uint2 rr = make_uint2(0u, 0u);
+      const uint32_t v = ent.x;
+      if (g < total && ((live >> own) & 1u)) {
+        const int64_t t = (int64_t)W.val[own] + ent.y;
+        if (t >= R.lb && t < R.ub_eff) {  // in the window [lb - d, ub - d)
           C.trav += 1;
-          const uint32_t nd = du + ent.y;  // < min(ub, 2^32 - 1) by the window
-          if (nd < __ldcg(&A.dist[v])) {
-            const uint32_t old = atomicMin(&A.dist[v], nd);
-            ok = nd < old;
-            first = ok && old == EIC_INF;
-          }
+          nd = (uint32_t)t;
+          const uint32_t old = atomicMin(&A.dist[v], nd);
+          rr = row_of(A.G, v);
+          prefetch_l2(&A.G.adj[rr.x]);
+          ok = nd < old;
+          first = ok && old == EIC_INF;
         }
       }
       C.improved += ok ? 1 : 0;
-      // into the local queue while it has room, else into the next round's queue (SAP)
-      const uint32_t m = __ballot_sync(EIC_FULL_MASK, ok);
-      const uint32_t cnt = __popc(m);
-      if (cnt && cnt <= kWarpStage - (lt - lh)) {
-        if (ok) lq[(lt + __popc(m & ((1u << lane) - 1u))) & (kWarpStage - 1)] = v;
-        lt += cnt;
-      } else if (cnt) {
-        bool sap = false;
-        if (ok) {
-          const uint32_t bit = 1u << (v & 31);
-          sap = !(atomicOr(&R.fbits[v >> 5], bit) & bit);
+      // into the local queue while it has room, else into the next round's queue (SAP); leaves are not relaxed from
+      const bool go = ok && rr.y > 1;
+      const uint32_t m = __ballot_sync(EIC_FULL_MASK, go);
+      if (m) {
+        uint32_t pos = 0;
+        if (lane == 0) pos = atomicAdd(&fcnt[wave], (uint32_t)__popc(m));
+        pos = __shfl_sync(EIC_FULL_MASK, pos, 0) + __popc(m & ((1u << lane) - 1u));
+        if (go && pos < room) fq[(lt + pos) & (kFuseQueue - 1)] = make_uint4(v, nd, rr.x, rr.y);
+        const bool over = go && pos >= room;
+        if (__any_sync(EIC_FULL_MASK, over)) {
+          const bool sap = over && claim_bit(R, v);
+          const uint32_t slot = warp_append(sap, R.qcnt_out);
+          if (sap) __stcg(&R.qout[slot], v);
         }
-        const uint32_t slot = warp_append(sap, R.qcnt_out);
-        if (sap) __stcg(&R.qout[slot], v);
       }
       warp_push(Fw, first, v);
-      __syncwarp();
     }
+    group_sync();  // the wave's pushes are complete
+    lt += min(fcnt[wave], room);
+    if (gw == 0 && lane == 0) fcnt[wave == 0 ? 2 : wave - 1] = 0;  // read by all before this barrier, next used two waves on
+    wave = wave == 2 ? 0 : wave + 1;
   }
   warp_flush(Fw);
   tl_block(A, 6, R.rid);
@@ -1463,7 +1513,8 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
         c->tcnt[(L.rid + 1) % 3] = 0;
         c->work[(L.rid + 1) % 3] = 0;
       }
-      {  // the other bitmap served round rid-1 and is next used in round rid+1: clear it now
+      if (L.cur_cnt) {  // the other bitmap served round rid-1 (which set a bit per vertex it queued) and is
+                        // next used in round rid+1: clear it now
         uint32_t* other = A.fbits + ((L.rid + 1) & 1u) * A.fwords;
         for (uint32_t wi = qb * blockDim.x + threadIdx.x; wi < A.fwords; wi += A.nb * blockDim.x)
           __stcg(&other[wi], 0u);
