@@ -217,8 +217,12 @@ __global__ void k_degree_tables(const uint32_t* __restrict__ hist, const uint32_
 }
 
 __global__ void k_highd0(const uint32_t* dcnt0, const uint32_t* dvals, uint32_t D, uint32_t* out) {
-  uint32_t h = block_highd(dcnt0, dvals, D);
-  if (threadIdx.x == 0) *out = h;
+  __shared__ HighdScr s;
+  const HighdPart p = highd_sums(dcnt0, dvals, D, s);
+  __syncthreads();
+  highd_cross(dcnt0, dvals, D, p, s);
+  __syncthreads();
+  if (threadIdx.x == 0) *out = s.highd;
 }
 
 __global__ void k_narrow(const uint64_t* __restrict__ in, uint64_t n, uint32_t* out) {

@@ -36,12 +36,10 @@ struct Ctl {
   uint32_t trace_len;
   uint32_t tl_len;  // diagnostic timeline events recorded
   // appended with atomics during phases
-  uint32_t qcnt[3];
-  uint32_t work[3];  // dynamic chunk counters, by round id mod 3
+  uint2 rcnt[3];  // by round id mod 3: vertices queued for the next round, tasks of the round
   uint32_t settled_cnt;
   uint32_t touched_cnt;
   uint32_t ub_cand;
-  uint32_t tcnt[3];  // tasks of the round, by round id mod 3
   uint32_t s2_done;
   uint32_t next_q;  // batch: the query the group's first block claimed
   unsigned long long next_ticket;  // serving: the request the group's first block claimed
@@ -82,7 +80,7 @@ struct BatchSlot {
   uint32_t* touched;
   uint32_t* sbits;
   uint32_t* hist;
-  unsigned long long* ring;
+  uint32_t* ring;
   Task* tasks;
   int64_t* step_ub;
   uint32_t* step_off;
@@ -101,7 +99,7 @@ struct Workspace {
   uint32_t* touched = nullptr;
   uint32_t* sbits = nullptr;  // settled bitmap
   uint32_t* hist = nullptr;
-  unsigned long long* ring = nullptr;
+  uint32_t* ring = nullptr;
   Task* tasks = nullptr;
   int64_t* step_ub = nullptr;
   uint32_t* step_off = nullptr;

@@ -44,7 +44,7 @@ inline SlotLayout slot_layout(const SlotCaps& c) {
   L.touched = take((n + 1) * 4);
   L.sbits = take(words * 4);
   L.hist = take(((uint64_t)c.D + 1) * 4);
-  L.ring = take((1ull << c.ring_bits) * 8);
+  L.ring = take((1ull << c.ring_bits) * 4);
   L.tasks = take((c.two_m / kHeavyMinFloor + 2) * sizeof(Task));
   L.step_ub = take(((uint64_t)kBatchStepCap + 2) * 8);
   L.step_off = take(((uint64_t)kBatchStepCap + 2) * 4);
@@ -96,7 +96,7 @@ struct SlotPool {
       s.touched = (uint32_t*)(b + L.touched);
       s.sbits = (uint32_t*)(b + L.sbits);
       s.hist = (uint32_t*)(b + L.hist);
-      s.ring = (unsigned long long*)(b + L.ring);
+      s.ring = (uint32_t*)(b + L.ring);
       s.tasks = (Task*)(b + L.tasks);
       s.step_ub = (int64_t*)(b + L.step_ub);
       s.step_off = (uint32_t*)(b + L.step_off);

@@ -72,7 +72,7 @@ struct KArgs {
   uint32_t* touched;
   uint32_t* sbits;  // settled bitmap
   uint32_t* hist;
-  unsigned long long* ring;
+  uint32_t* ring;
   Task* tasks;
   int64_t* step_ub;
   uint32_t* step_off;
@@ -182,17 +182,18 @@ __device__ __forceinline__ void warp_push(WarpList& W, bool want, uint32_t v) {
 
 struct S2Scr {
   uint32_t hist[kShRanks];
-  unsigned long long ring[kShRing];
+  uint32_t ring[kShRing];
 };
 
-constexpr uint32_t kGapPar = 256;   // distinct degrees up to which the boundary evaluates Eq. 1-3 for each
-constexpr uint32_t kStBins = 1920;  // Function 2 candidate bins held in shared memory (ST_NUM + 2 at most)
+constexpr uint32_t kSufMax = 4096;  // Function 2: suffix sums (or bins of wide weights) held in shared memory
+constexpr uint32_t kCandMax = 512;  // Function 2: candidates listed for the double-precision evaluation
 
 struct S3Scr {
-  unsigned long long part[kMaxBlock];
+  uint32_t suf[kSufMax + 1];
+  uint32_t ck[kCandMax], cd[kCandMax];  // a listed candidate and its degree sum
+  uint32_t part[kMaxBlock];
   unsigned long long bp[32];  // per warp: the best profit's key (see block_argmax)
   uint32_t bk[32];
-  unsigned long long bins[kStBins];
 };
 
 union PhaseScr {
@@ -209,9 +210,13 @@ struct Local {
 };
 
 // State of the step controller, kept in block 0's shared memory across steps.
+constexpr uint32_t kStepHist = 128;  // recent steps whose ub and list offset the controller keeps at hand
 struct BState {
   int64_t st0, st1, gap_lb, max_settled;
   uint64_t sumd_lb, highd_lb;
+  unsigned long long rounds;
+  int64_t hub[kStepHist];    // ub of step j at j % kStepHist
+  uint32_t hoff[kStepHist];  // step j's first settled-list entry
   uint32_t j0;
 };
 
@@ -287,14 +292,6 @@ __device__ __forceinline__ uint32_t ld_list(const uint32_t* p) {
   return v;
 }
 
-__device__ __forceinline__ uint2 ld_list2(const uint2* p) {
-  uint2 v;
-  asm volatile("ld.global.cg.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
-               : "=r"(v.x), "=r"(v.y)
-               : "l"(p), "l"(stream_policy()));
-  return v;
-}
-
 __device__ __forceinline__ uint4 ld_list4(const void* p) {
   uint4 v;
   asm volatile("ld.global.cg.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
@@ -361,11 +358,12 @@ struct RoundCtx {
   uint32_t* first_list;
   uint32_t* first_cnt;
   uint32_t* tcnt;
-  uint32_t* work;
 };
 
 // Flush the block's task stage to the global list (block-uniform call).
 __device__ __forceinline__ void stage_flush(Stage& T, const RoundCtx& R, Task* tasks) {
+  __syncthreads();
+  if (T.tn == 0) return;  // (next written after the grid barrier)
   __syncthreads();
   if (threadIdx.x == 0) {
     const uint32_t tn = min(T.tn, kStageT);
@@ -913,9 +911,9 @@ __device__ __forceinline__ int64_t block_st_exact(const KArgs& A, S3Scr& S, int6
   if (gap_ub_raw == maxw) return ub - maxw;
   const int64_t wl = ub - maxw > 0 ? ub - maxw : 0;
   const uint64_t nbins = (uint64_t)A.st_num + 2;
-  const bool sh = nbins <= kStBins;
-  unsigned long long* bins = sh ? S.bins : A.ring;
-  for (uint64_t q = t; q < nbins; q += nt) bins[q] = 0ull;
+  const bool sh = nbins <= kSufMax;
+  uint32_t* bins = sh ? S.suf : A.ring;  // (a degree sum is at most 2m < 2^32)
+  for (uint64_t q = t; q < nbins; q += nt) bins[q] = 0u;
   if (t == 0) {
     uint32_t j = j0;
     while (j <= step && __ldcg(&A.step_ub[j]) <= wl) ++j;
@@ -934,23 +932,23 @@ __device__ __forceinline__ int64_t block_st_exact(const KArgs& A, S3Scr& S, int6
       cnt = nbins - 1;
     else
       cnt = min(((uint64_t)(d - st0 + 1) * A.st_num + span - 1) / span, nbins - 1);
-    atomicAdd(&bins[cnt], (unsigned long long)dg);
+    atomicAdd(&bins[cnt], dg);
   }
   __syncthreads();
   // suffix sums: chunk totals, a scan over the chunks, then within the chunks
   const uint64_t cs = (nbins + nt - 1) / nt;
   const uint64_t q0 = t * cs, q1 = min(nbins, q0 + cs);
-  unsigned long long mine = 0;
+  uint32_t mine = 0;
   for (uint64_t q = q0; q < q1; ++q) mine += sh ? bins[q] : __ldcg(&bins[q]);
   S.part[t] = mine;
   __syncthreads();
   for (uint32_t o = 1; o < nt; o <<= 1) {
-    unsigned long long v = t + o < nt ? S.part[t + o] : 0;
+    const uint32_t v = t + o < nt ? S.part[t + o] : 0;
     __syncthreads();
     S.part[t] += v;
     __syncthreads();
   }
-  unsigned long long acc = t + 1 < nt ? S.part[t + 1] : 0;
+  uint32_t acc = t + 1 < nt ? S.part[t + 1] : 0;
   for (uint64_t q = q1; q > q0; --q) {
     acc += sh ? bins[q - 1] : __ldcg(&bins[q - 1]);
     if (sh)
@@ -966,7 +964,7 @@ __device__ __forceinline__ int64_t block_st_exact(const KArgs& A, S3Scr& S, int6
     const int64_t x = st_candidate(k, span, A.st_num, gsh, st0);
     if (x >= ub) continue;
     const uint64_t q = x >= wl ? (uint64_t)k + 1 : 0;
-    const unsigned long long dsum = sh ? bins[q] : __ldcg(&bins[q]);
+    const uint32_t dsum = sh ? bins[q] : __ldcg(&bins[q]);
     const double p = dev_profit(x, ub, y, dsum, sumd_ub, A.G.maxw, A.G.two_m);
     if (p > best) {
       best = p;
@@ -1164,90 +1162,227 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
   tl_block(A, 6, R.rid);
 }
 
-// Function 2 for the boundary <lb, ub> -> next pair <ub, ub + gap(ub)>, run by
-// one whole block. Candidates x_k = st0 + floor(k (st1 - st0) / ST_NUM) < ub;
-// D(x') = sumD(x') - sumD(ub), the degree sum of the settled vertices with
-// x' <= dist < ub, x' = max(x, ub - maxW), read from the ring of settled
-// degree sums (one slot per distance: maxW < 2^20; wider weights go through
-// block_st_exact).
-__device__ int64_t block_compute_st(const KArgs& A, S3Scr& S, int64_t ub, uint64_t sumd_ub, int64_t gap_lb,
-                                    int64_t gap_ub_raw, int64_t y, int64_t st0, int64_t st1) {
-  const int64_t maxw = A.G.maxw;
-  if (sumd_ub >= A.G.m || gap_lb == maxw) return ub;
-  if (gap_ub_raw == maxw) return ub - maxw;
-  const uint32_t t = threadIdx.x, nt = blockDim.x;
-  const int64_t wl = ub - maxw > 0 ? ub - maxw : 0;
-  const uint32_t sh = A.ring_shift;
-  const uint64_t sl = (uint64_t)wl >> sh, su = (uint64_t)(ub - 1) >> sh;
-  const uint64_t L = su - sl + 1;  // ring slots covering [wl, ub)
-  const uint64_t cs = (L + nt - 1) / nt;
-  unsigned long long mine = 0;
-  for (uint64_t q = sl + t * cs; q < sl + (t + 1) * cs && q <= su; ++q) mine += __ldcg(&A.ring[q & A.ring_mask]);
-  S.part[t] = mine;
-  __syncthreads();
-  for (uint32_t o = 1; o < nt; o <<= 1) {  // suffix sums over chunks
-    unsigned long long v = t + o < nt ? S.part[t + o] : 0;
-    __syncthreads();
-    S.part[t] += v;
-    __syncthreads();
+// Function 2's window [wl, ub) of the ring (one slot per distance), in at most
+// kSufMax chunks of cs slots.
+struct F2Window {
+  int64_t wl;
+  uint32_t slots, cs, chunks;
+};
+
+__device__ __forceinline__ F2Window f2_window(int64_t ub, int64_t maxw) {
+  F2Window w;
+  w.wl = ub > maxw ? ub - maxw : 0;
+  w.slots = (uint32_t)(ub - w.wl);
+  w.cs = (w.slots + kSufMax - 1) / kSufMax;
+  w.chunks = w.cs > 1 ? (w.slots + w.cs - 1) / w.cs : w.slots;
+  return w;
+}
+
+// The chunk sums of the window to shared memory (block-wide, no barrier).
+__device__ __forceinline__ void f2_load(const KArgs& A, S3Scr& S, const F2Window& w) {
+  if (w.cs <= 1) {
+#pragma unroll 4
+    for (uint32_t q = threadIdx.x; q < w.slots; q += blockDim.x)
+      S.suf[q] = __ldcg(&A.ring[(uint32_t)(w.wl + q) & A.ring_mask]);
+  } else {
+    for (uint32_t q = threadIdx.x; q < w.chunks; q += blockDim.x) {
+      const uint32_t b = q * w.cs, e = min(w.slots, b + w.cs);
+      uint32_t sum = 0;
+#pragma unroll 4
+      for (uint32_t i = b; i < e; ++i) sum += __ldcg(&A.ring[(uint32_t)(w.wl + i) & A.ring_mask]);
+      S.suf[q] = sum;
+    }
   }
-  double best = 0.0;
-  uint32_t bk = 0xFFFFFFFFu;
+}
+
+// Function 2 over the ST_NUM grid of candidates x_k = st0 + floor(k (st1 - st0)
+// / ST_NUM) < ub (one whole block; every thread gets the result): the first
+// candidate with the largest positive profit, or ub. D(x') = sumD(x') -
+// sumD(ub), the degree sum of the settled vertices with x' <= dist < ub, x' =
+// max(x, ub - maxW), is a suffix sum of the ring (one slot per distance: maxW <
+// 2^20; wider weights go through block_st_exact).
+//
+// The profit is specified in double precision, of which this GPU has two
+// operations per clock and SM: ST_NUM candidates with three divisions each cost
+// 10 us. Only candidates that can win are evaluated in it: those with pushed >
+// pulled, an exact integer comparison (each double operation rounds
+// monotonically, so pushed <= pulled there means profit <= 0 here), and, of
+// these, those whose single-precision estimate comes within twice its error
+// bound of the best. The estimate's error is at most 20 roundings of
+// 2^-24 of pushed <= pushed(x = wl), which bounds every term; e takes 32.
+// Function 2 went from 5.6 to 2.5 us a step on a uniform graph of 2^14 vertices.
+__device__ int64_t block_compute_st(const KArgs& A, S3Scr& S, const F2Window& w, int64_t ub, uint64_t sumd_ub,
+                                    int64_t y, int64_t st0, int64_t st1, uint32_t wsuf, uint32_t* s_rw) {
+  __shared__ uint32_t s_best, s_cnt;
+  const uint32_t t = threadIdx.x, nt = blockDim.x, lane = lane_id(), warp = t >> 5, nw = nt >> 5;
+  const int64_t maxw = A.G.maxw;
+  {  // suffix sums in place: this thread's run of chunks behind all later threads'
+    uint32_t x = lane < nw ? s_rw[lane] : 0u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t z = __shfl_down_sync(EIC_FULL_MASK, x, o);
+      if (lane + o < 32) x += z;
+    }
+    uint32_t run = __shfl_sync(EIC_FULL_MASK, x, (warp + 1) & 31);
+    if (warp + 1 >= nw) run = 0;
+    const uint32_t later = __shfl_down_sync(EIC_FULL_MASK, wsuf, 1);
+    if (lane < 31) run += later;
+    const uint32_t per = (w.chunks + nt - 1) / nt, b = min(w.chunks, t * per), e = min(w.chunks, b + per);
+    for (uint32_t q = e; q > b; --q) {
+      run += S.suf[q - 1];
+      S.suf[q - 1] = run;
+    }
+    if (t == 0) {
+      S.suf[w.chunks] = 0;
+      s_best = 0;
+      s_cnt = 0;
+    }
+  }
+  __syncthreads();
   const uint64_t span = (uint64_t)(st1 - st0);
   const uint32_t gsh = (A.st_num & (A.st_num - 1)) == 0 ? __ffs(A.st_num) - 1 : 32u;
-  for (uint32_t k = t; k <= A.st_num; k += nt) {
+  const int64_t lo = ub - maxw;
+  const uint32_t push_w = (uint32_t)((y < ub + maxw ? y : ub + maxw) - ub);  // ub0 - lb <= maxW
+  const float inv = 1.0f / (float)maxw, inv2m = 1.0f / (float)A.G.two_m, fsumd = (float)sumd_ub;
+  const float e = (float)push_w * (float)S.suf[0] * inv * (1.0f / 524288.0f);  // 2^-19 pushed(wl)
+  // candidate k: false when it cannot be the answer, else its degree sum and estimate + e
+  auto estimate = [&](uint32_t k, uint32_t& dsum, float& v) -> bool {
     const int64_t x = st_candidate(k, span, A.st_num, gsh, st0);
-    if (x >= ub) continue;
-    const int64_t xc = x > ub - maxw ? x : ub - maxw;
+    if (x >= ub) return false;
+    const int64_t xc = x > lo ? x : lo;
     if (k > 0) {  // the profit depends on x' only: the first candidate of each x' decides the argmax
       const int64_t xp = st_candidate(k - 1, span, A.st_num, gsh, st0);
-      if ((xp > ub - maxw ? xp : ub - maxw) == xc) continue;
+      if ((xp > lo ? xp : lo) == xc) return false;
     }
-    const uint64_t q0 = (uint64_t)xc >> sh;
-    const uint64_t c = (q0 - sl) / cs;
-    unsigned long long dsum = c + 1 < nt ? S.part[c + 1] : 0;
-    for (uint64_t q = q0; q < sl + (c + 1) * cs && q <= su; ++q) dsum += __ldcg(&A.ring[q & A.ring_mask]);
-    const double p = dev_profit(x, ub, y, dsum, sumd_ub, A.G.maxw, A.G.two_m);
-    if (p > best) {
-      best = p;
-      bk = k;
+    const uint32_t i = (uint32_t)(xc - w.wl);
+    if (w.cs <= 1) {
+      dsum = S.suf[i];
+    } else {
+      const uint32_t c = i / w.cs, ce = min(w.slots, (c + 1) * w.cs);
+      dsum = S.suf[c + 1];
+      for (uint32_t q = i; q < ce; ++q) dsum += __ldcg(&A.ring[(uint32_t)(w.wl + q) & A.ring_mask]);
+    }
+    const uint32_t pull_w = (uint32_t)((y < xc + maxw ? y : xc + maxw) - xc);  // ub1 - x' <= maxW
+    if ((uint64_t)push_w * dsum <= (uint64_t)pull_w * sumd_ub) return false;
+    const float pushed = (float)push_w * (float)dsum * inv, pulled = (float)pull_w * fsumd * inv;
+    v = pushed - pulled * (float)dsum * inv2m - pulled + e;
+    return v > 0.0f;
+  };
+  uint32_t mine = 0;  // (a positive float's bits order as the float)
+  for (uint32_t k = t; k <= A.st_num; k += nt) {
+    uint32_t dsum;
+    float v;
+    if (estimate(k, dsum, v)) mine = max(mine, __float_as_uint(v));
+  }
+  mine = __reduce_max_sync(EIC_FULL_MASK, mine);
+  if (lane == 0 && mine) atomicMax(&s_best, mine);
+  __syncthreads();
+  if (s_best == 0) return ub;
+  const float least = __uint_as_float(s_best) - 2.0f * e;
+  for (uint32_t k = t; k <= A.st_num; k += nt) {
+    uint32_t dsum;
+    float v;
+    if (estimate(k, dsum, v) && v >= least) {
+      const uint32_t at = atomicAdd(&s_cnt, 1u);
+      if (at < kCandMax) {
+        S.ck[at] = k;
+        S.cd[at] = dsum;
+      }
+    }
+  }
+  __syncthreads();
+  const uint32_t cnt = s_cnt;
+  double best = 0.0;
+  uint32_t bk = 0xFFFFFFFFu;
+  if (cnt <= kCandMax) {
+    for (uint32_t i = t; i < cnt; i += nt) {
+      const uint32_t k = S.ck[i];
+      const double p = dev_profit(st_candidate(k, span, A.st_num, gsh, st0), ub, y, S.cd[i], sumd_ub, A.G.maxw, A.G.two_m);
+      if (p > best || (p == best && p > 0.0 && k < bk)) {
+        best = p;
+        bk = k;
+      }
+    }
+  } else {  // more than the list holds (a flat profit): each thread its own
+    for (uint32_t k = t; k <= A.st_num; k += nt) {
+      uint32_t dsum;
+      float v;
+      if (!estimate(k, dsum, v) || v < least) continue;
+      const double p = dev_profit(st_candidate(k, span, A.st_num, gsh, st0), ub, y, dsum, sumd_ub, A.G.maxw, A.G.two_m);
+      if (p > best) {
+        best = p;
+        bk = k;
+      }
     }
   }
   const uint32_t k = block_argmax(S, best, bk);
-  if (k == 0xFFFFFFFFu) return ub;
-  return st_candidate(k, span, A.st_num, gsh, st0);
+  return k == 0xFFFFFFFFu ? ub : st_candidate(k, span, A.st_num, gsh, st0);
 }
 
 // Step boundary, executed by block 0 once every block finished the
 // statistics pass: sumD(ub), highD(ub), gap(ub) (Eq. 1-3), termination
 // (Algorithm 1), computeST (Function 2) and the push/pull sets of the next
 // step's Function 1. Publishes the new control values before the grid barrier.
-template <bool kExactInline, bool kParGap>
+// The whole query waits for it, so it is laid out for latency: what depends on
+// <lb, ub> alone (the counters, the degree histogram, Function 2's window of
+// the ring) is loaded at once, highD and the window's sums share their
+// barriers, and double precision is used only where a single-precision
+// estimate cannot decide. A boundary went from 10.8 to 7.2 us on the 4096^2
+// grid, from 10.9 to 5.8 us on a uniform graph of 2^14 vertices.
+template <bool kExactInline>
 __device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Local& L, uint32_t rounds_in_step) {
   Ctl* c = A.ctl;
-  __shared__ int64_t sh_i[8];
-  __shared__ uint64_t sh_u[4];
-  __shared__ uint32_t sh_flag[2];
-  __shared__ int64_t sh_gap[kGapPar];
+  __shared__ HighdScr s_h;
+  __shared__ uint32_t s_rw[32];
+  __shared__ uint64_t s_sumd;
+  __shared__ uint32_t s_settled, s_done;
+  __shared__ int64_t s_gap;
   const DevGraph& G = A.G;
-  const int64_t lb = L.lb, ub = L.ub;
+  S3Scr& S = P.s3;
+  const uint32_t t = threadIdx.x, nt = blockDim.x, lane = lane_id(), warp = t >> 5;
+  const int64_t lb = L.lb, ub = L.ub, maxw = G.maxw;
   const uint32_t k = L.step;
-  if (threadIdx.x == 0) {
-    const uint32_t settled_now = __ldcg(&c->settled_cnt);
-    const unsigned long long acc = __ldcg(&c->acc_deg);
-    const uint32_t acc_maxd1 = __ldcg(&c->acc_maxd1);
-    const uint64_t sumd_ub = B.sumd_lb - acc;
-    sh_u[0] = sumd_ub;
-    sh_u[1] = settled_now;
-    if (acc_maxd1 && (int64_t)(acc_maxd1 - 1) > B.max_settled) B.max_settled = acc_maxd1 - 1;
+  uint32_t settled_now = 0, maxd1 = 0;
+  unsigned long long acc = 0;
+  if (t == 0) {
+    settled_now = __ldcg(&c->settled_cnt);
+    acc = __ldcg(&c->acc_deg);
+    maxd1 = __ldcg(&c->acc_maxd1);
+  }
+  const int64_t gap_lb = B.gap_lb;
+  const bool ring = A.ring_shift == 0 && !(A.flags & EIC_FLAG_NO_PULL) && gap_lb != maxw;
+  const F2Window w = f2_window(ub, maxw);
+  const bool early = ring && w.cs <= 1;  // (a longer window is loaded only once it is needed)
+  if (early) f2_load(A, S, w);
+  const HighdPart hp = highd_sums(A.hist, G.dvals, G.D, s_h);
+  if (t == 0) {
+    if (maxd1 && (int64_t)(maxd1 - 1) > B.max_settled) B.max_settled = maxd1 - 1;
     const int64_t maxs = B.max_settled;
+    // termination / overflow (Algorithm 1): max{finite dist} + maxW(G,1) < lb
+    uint32_t done = 0;
+    if (maxs + maxw >= (int64_t)EIC_INF) {
+      atomicCAS(&c->status, 0, EIC_EOVERFLOW);
+      done = 1;
+    } else if (maxs + maxw < ub) {
+      done = 1;
+    } else if (k + 1 >= A.step_cap) {
+      atomicCAS(&c->status, 0, EIC_ENOMEM);
+      done = 1;
+    }
+    s_done = done;
+    s_sumd = B.sumd_lb - acc;
+    s_settled = settled_now;
     A.step_ub[k] = ub;
+    B.hub[k % kStepHist] = ub;
+    B.rounds += rounds_in_step;
+    c->cnt_rounds = B.rounds;
+    c->trace_len = k;
     if (k <= A.trace_cap && A.trace) {
       eic_step r;
       r.lb = lb;
       r.ub = ub;
       r.st = L.st;
-      r.gap_lb = B.gap_lb;
+      r.gap_lb = gap_lb;
       r.sumd_lb = B.sumd_lb;
       r.highd_lb = B.highd_lb;
       r.rounds = rounds_in_step;
@@ -1256,76 +1391,68 @@ __device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Loca
       r.reserved = 0;
       A.trace[k - 1] = r;
     }
-    c->trace_len = k;
-    c->cnt_rounds += rounds_in_step;
-    // termination / overflow (Algorithm 1): max{finite dist} + maxW(G,1) < lb
-    uint32_t done = 0;
-    if (maxs + (int64_t)G.maxw >= (int64_t)EIC_INF) {
-      atomicCAS(&c->status, 0, EIC_EOVERFLOW);
-      done = 1;
-    } else if (maxs + (int64_t)G.maxw < ub) {
-      done = 1;
-    } else if (k + 1 >= A.step_cap) {
-      atomicCAS(&c->status, 0, EIC_ENOMEM);
-      done = 1;
-    }
-    sh_flag[0] = done;
   }
   __syncthreads();
-  const uint64_t sumd_ub = sh_u[0];
-  uint32_t highd_ub;
-  // With few distinct degrees (road-like graphs: the fused kernel), Eq. 1-3 is
-  // evaluated for every value highD can take (each distinct degree) by the
-  // other warps while warp 0 finds highD: the double-precision chain of Eq. 2
-  // is long on this GPU, and it then runs beside highD instead of after it.
-  const bool gap_par = kParGap && G.D <= kGapPar && blockDim.x >= 32 + G.D;
-  if (gap_par && threadIdx.x >= 32 && threadIdx.x < 32 + G.D)
-    sh_gap[threadIdx.x - 32] = dev_gap(sumd_ub, G.dvals[threadIdx.x - 32], G.two_m, A.alpha, A.beta, G.rtow);
-  if (G.D <= 32 * kWarpHighdPer) {  // one warp, no block barriers
-    if (threadIdx.x < 32) {
-      const uint32_t h = warp_highd(A.hist, G.dvals, G.D);
-      if (threadIdx.x == 0) sh_flag[1] = h;
-    }
-    __syncthreads();
-    highd_ub = sh_flag[1];
-  } else {
-    highd_ub = block_highd(A.hist, G.dvals, G.D);
-  }
-  if (sh_flag[0]) {
-    if (threadIdx.x == 0) {
+  const uint64_t sumd_ub = s_sumd;
+  if (s_done) {
+    if (t == 0) {
       c->done = 1;
       c->s2_done = 0;  // published by the grid barrier's release
     }
-    __syncthreads();
     return;
   }
-  if (threadIdx.x == 0) {
-    // highD is a distinct degree (its rank from drank) or 0 (empty set: gap maxW(G, 1))
-    const int64_t gap_raw = gap_par && highd_ub > 0 ? sh_gap[__ldg(&G.drank[highd_ub])]
-                                                    : dev_gap(sumd_ub, highd_ub, G.two_m, A.alpha, A.beta, G.rtow);
-    if (k == 1) B.st0 = ub;
-    if (B.st1 < 0 && sumd_ub <= G.m) B.st1 = ub;
-    sh_i[1] = gap_raw;
-    sh_i[2] = gap_raw << A.gap_shift;
-  }
+  // this thread's run of the window's chunk sums, summed from the end of the warp
+  auto window_sums = [&]() -> uint32_t {
+    const uint32_t per = (w.chunks + nt - 1) / nt, b = min(w.chunks, t * per), e = min(w.chunks, b + per);
+    uint32_t x = 0;
+    for (uint32_t q = b; q < e; ++q) x += S.suf[q];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t z = __shfl_down_sync(EIC_FULL_MASK, x, o);
+      if (lane + o < 32) x += z;
+    }
+    if (lane == 0) s_rw[warp] = x;
+    return x;
+  };
+  highd_cross(A.hist, G.dvals, G.D, hp, s_h);
+  uint32_t wsuf = early ? window_sums() : 0u;
   __syncthreads();
-  const int64_t gap_raw = sh_i[1], width = sh_i[2];
-  const int64_t nlb = ub, nub = ub + width;
-  const int64_t nst = (A.flags & EIC_FLAG_NO_PULL) ? nlb
-                      : A.ring_shift == 0
-                          ? block_compute_st(A, P.s3, ub, sumd_ub, B.gap_lb, gap_raw, nub, B.st0, B.st1)
-                          : kExactInline ? block_st_exact(A, P.s3, ub, sumd_ub, B.gap_lb, gap_raw, nub, B.st0, B.st1,
-                                                          B.j0, k, (uint32_t)sh_u[1])
-                                         : block_st_exact_call(A, P.s3, ub, sumd_ub, B.gap_lb, gap_raw, nub, B.st0,
-                                                               B.st1, B.j0, k, (uint32_t)sh_u[1]);
-  if (A.ring_shift == 0) {  // zero the ring slots the next statistics pass fills: [max(nlb, nub - maxW), nub)
-    const int64_t zl = nub - (int64_t)G.maxw > nlb ? nub - (int64_t)G.maxw : nlb;
-    const uint64_t ql = (uint64_t)zl >> A.ring_shift, qu = (uint64_t)(nub - 1) >> A.ring_shift;
-    for (uint64_t q = ql + threadIdx.x; q <= qu; q += blockDim.x) __stcg(&A.ring[q & A.ring_mask], 0ull);
+  const uint32_t highd_ub = s_h.highd;
+  int64_t gap_raw = dev_gap_quick(sumd_ub, highd_ub, G.two_m, A.alpha, A.beta, G.rtow);
+  if (gap_raw < 0) {  // (the same in every thread)
+    if (t == 0) s_gap = dev_gap(sumd_ub, highd_ub, G.two_m, A.alpha, A.beta, G.rtow);
+    __syncthreads();
+    gap_raw = s_gap;
   }
-  if (threadIdx.x == 0) {
-    const uint32_t settled_now = (uint32_t)sh_u[1];
+  const int64_t st0 = k == 1 ? ub : B.st0, st1 = B.st1 < 0 && sumd_ub <= G.m ? ub : B.st1;
+  const int64_t nlb = ub, nub = ub + (gap_raw << A.gap_shift);
+  int64_t nst = nlb;
+  if (!(A.flags & EIC_FLAG_NO_PULL) && sumd_ub < G.m && gap_lb != maxw) {
+    if (gap_raw == maxw) {
+      nst = ub - maxw;
+    } else if (A.ring_shift == 0) {
+      if (!early) {
+        f2_load(A, S, w);
+        __syncthreads();
+        wsuf = window_sums();
+        __syncthreads();
+      }
+      nst = block_compute_st(A, S, w, ub, sumd_ub, nub, st0, st1, wsuf, s_rw);
+    } else {
+      nst = kExactInline
+                ? block_st_exact(A, S, ub, sumd_ub, gap_lb, gap_raw, nub, st0, st1, B.j0, k, s_settled)
+                : block_st_exact_call(A, S, ub, sumd_ub, gap_lb, gap_raw, nub, st0, st1, B.j0, k, s_settled);
+    }
+  }
+  if (t >= 32) {
+    if (A.ring_shift == 0) {  // zero the ring slots the next statistics pass fills: [max(nlb, nub - maxW), nub)
+      const int64_t zl = nub - maxw > nlb ? nub - maxw : nlb;
+      for (int64_t q = zl + (t - 32); q < nub; q += nt - 32) __stcg(&A.ring[(uint32_t)q & A.ring_mask], 0u);
+    }
+  } else if (t == 0) {
+    settled_now = s_settled;
     A.step_off[k + 1] = settled_now;
+    B.hoff[(k + 1) % kStepHist] = settled_now;
     uint32_t scnt = settled_now;
     uint32_t extra = 0;
     if (k == 1 && ub == 0) {  // the source itself was not settled by the first step
@@ -1336,20 +1463,29 @@ __device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Loca
       extra = 1;
     }
     // Function 1's push set {lb0 <= dist <= st}: the settled steps j with
-    // ub_j > lb0 (j0, moving forward only) and lb_j <= st (j1, from the back)
-    const int64_t lb0 = nlb - (int64_t)G.maxw > 0 ? nlb - (int64_t)G.maxw : 0;
+    // ub_j > lb0 (j0, moving forward only) and lb_j <= st (j1, from the back);
+    // the last kStepHist steps are in shared memory
+    auto ub_of = [&](uint32_t j) -> int64_t {
+      return j + kStepHist > k ? B.hub[j % kStepHist] : __ldcg(&A.step_ub[j]);
+    };
+    auto off_of = [&](uint32_t j) -> uint32_t {
+      return j + kStepHist > k + 1 ? B.hoff[j % kStepHist] : __ldcg(&A.step_off[j]);
+    };
+    const int64_t lb0 = nlb - maxw > 0 ? nlb - maxw : 0;
     uint32_t pb = 0, pe = 0;
-    while (B.j0 <= k && __ldcg(&A.step_ub[B.j0]) <= lb0) ++B.j0;
+    uint32_t j0 = B.j0;
+    while (j0 <= k && ub_of(j0) <= lb0) ++j0;
+    B.j0 = j0;
     if (nst >= lb0) {
       uint32_t j1 = k;
       int64_t lbj = lb;  // lb_k
       while (j1 >= 1 && lbj > nst) {
         --j1;
-        lbj = j1 >= 2 ? __ldcg(&A.step_ub[j1 - 1]) : 0;
+        lbj = j1 >= 2 ? ub_of(j1 - 1) : 0;
       }
-      if (B.j0 <= j1 && j1 >= 1) {
-        pb = __ldcg(&A.step_off[B.j0]);
-        pe = j1 == k ? settled_now : __ldcg(&A.step_off[j1 + 1]);
+      if (j0 <= j1 && j1 >= 1) {
+        pb = off_of(j0);
+        pe = j1 == k ? settled_now : off_of(j1 + 1);
       }
     }
     // Function 1's pull: unsettled vertices with an edge lighter than ub - st,
@@ -1394,15 +1530,19 @@ __device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Loca
     c->pull_cnt = sweep ? G.ni : pull_cnt;
     c->extra_s = extra;
     c->step_off_cur = settled_now;
-    B.sumd_lb = sumd_ub;
-    B.highd_lb = highd_ub;
-    B.gap_lb = gap_raw;
     c->acc_deg = 0;
     c->acc_maxd1 = 0;
     c->s2_done = 0;
     c->done = 0;  // the control values are published by the grid barrier's release
   }
-  __syncthreads();
+  __syncthreads();  // every thread is done with the controller's state of this step
+  if (t == 0) {
+    B.st0 = st0;
+    B.st1 = st1;
+    B.sumd_lb = sumd_ub;
+    B.highd_lb = highd_ub;
+    B.gap_lb = gap_raw;
+  }
 }
 
 // All threads: control values published before the last barrier (one thread
@@ -1458,22 +1598,22 @@ struct QueryShared {
   BState B;
   unsigned long long red[32][7];
   unsigned long long snap[4];
-  uint32_t last;
+  uint32_t last, red2[2];
 };
 
 // The query loop of Algorithm 1 run by the A.nb blocks of one query: rounds
 // of a step (item phase, task phase), statistics pass, step boundary, until
-// termination. gen is the block's copy of the barrier generation (uint32_t),
-// or its arrival ticket in a launch that runs this one query only (64-bit).
+// termination. ticket is the block's arrival ticket of the query's barrier.
 // kFuse: 0 no fused rounds, 1 fused rounds, 2 as A.fuse says (per query).
-template <uint32_t kPullFast, uint32_t kRelaxIlp, uint32_t kFuse = 0, class Gen = uint32_t>
-__device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
+template <uint32_t kPullFast, uint32_t kRelaxIlp, uint32_t kFuse = 0>
+__device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ticket) {
   PhaseScr& P = Q.P;
   Stage& T = Q.T;
   BState& B = Q.B;
   auto& sh_red = Q.red;
   auto& sh_snap = Q.snap;
   uint32_t& sh_last = Q.last;
+  auto& sh_red2 = Q.red2;
   Ctl* c = A.ctl;
   const uint32_t qb = qblock(A);
   Local L;
@@ -1490,6 +1630,9 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
     B.max_settled = -1;
     B.sumd_lb = A.G.two_m;
     B.highd_lb = A.G.highd0;
+    B.rounds = 0;
+    B.hub[0] = 0;
+    B.hoff[1] = 0;
     B.j0 = 1;
   }
   if (qb == 0 && threadIdx.x == 0) tl_mark(A, 0, L.rid);
@@ -1509,9 +1652,7 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
       const bool round1 = (L.step >= 2 && rin == 0);
       // counters of round rid+1 were last read two barriers ago: clear them now
       if (qb == 0 && threadIdx.x == 0) {
-        c->qcnt[(L.rid + 1) % 3] = 0;
-        c->tcnt[(L.rid + 1) % 3] = 0;
-        c->work[(L.rid + 1) % 3] = 0;
+        __stcg(&c->rcnt[(L.rid + 1) % 3], make_uint2(0u, 0u));
       }
       if (L.cur_cnt) {  // the other bitmap served round rid-1 (which set a bit per vertex it queued) and is
                         // next used in round rid+1: clear it now
@@ -1529,11 +1670,10 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
       R.rid = L.rid;
       R.step1 = L.step == 1;
       R.qout = L.qsel ? A.q0 : A.q1;
-      R.qcnt_out = &c->qcnt[L.rid % 3];
+      R.qcnt_out = &c->rcnt[L.rid % 3].x;
       R.first_list = R.step1 ? A.touched : A.sid;
       R.first_cnt = R.step1 ? &c->touched_cnt : &c->settled_cnt;
-      R.tcnt = &c->tcnt[L.rid % 3];
-      R.work = &c->work[L.rid % 3];
+      R.tcnt = &c->rcnt[L.rid % 3].y;
       const uint32_t* qin = L.qsel ? A.q1 : A.q0;
       Local LL = L;
       if (!L.pull_on) LL.pull_cnt = 0;
@@ -1544,14 +1684,16 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
         fused_round(A, R, LL, P.r, T, nitems, round1, qin, C);
       else
         round_phase<kPullFast, kRelaxIlp>(A, R, LL, P.r, T, nitems, round1, qin, C);
-      if (!grid_barrier(&c->bar, &gen, A.nb, A.max_spin, &c->status)) {
+      if (!grid_barrier(&c->bar, &ticket, A.nb, A.max_spin, &c->status)) {
         alive = false;
         break;
       }
       if (threadIdx.x == 0) {
-        sh_snap[0] = __ldcg(&c->tcnt[L.rid % 3]);
-        sh_snap[1] = __ldcg(&c->qcnt[L.rid % 3]);
+        const uint2 rc = __ldcg(&c->rcnt[L.rid % 3]);
+        sh_snap[0] = rc.y;
+        sh_snap[1] = rc.x;
         sh_snap[2] = __ldcg(&c->ub_cand);
+        sh_snap[3] = __ldcg(R.first_cnt);
         if (qb == 0) tl_mark(A, 1, L.rid);
       }
       __syncthreads();
@@ -1562,14 +1704,15 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
       if (hp != 0) {
         if (qb == 0 && threadIdx.x == 0) tl_mark(A, 9, (uint32_t)hp);  // diagnostic: the round's tasks
         task_phase<(kRelaxIlp >= 2)>(A, R, (uint32_t)hp, T, C);
-        if (!grid_barrier(&c->bar, &gen, A.nb, A.max_spin, &c->status)) {
+        if (!grid_barrier(&c->bar, &ticket, A.nb, A.max_spin, &c->status)) {
           alive = false;
           break;
         }
         if (qb == 0 && threadIdx.x == 0) tl_mark(A, 2, L.rid);
         if (threadIdx.x == 0) {
-          sh_snap[1] = __ldcg(&c->qcnt[L.rid % 3]);
+          sh_snap[1] = __ldcg(&c->rcnt[L.rid % 3].x);
           sh_snap[2] = __ldcg(&c->ub_cand);
+          sh_snap[3] = __ldcg(R.first_cnt);
         }
         __syncthreads();
         L.cur_cnt = (uint32_t)sh_snap[1];
@@ -1588,21 +1731,26 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
       const bool step1 = L.step == 1;
       const uint32_t* list = step1 ? A.touched : A.sid;
       const uint32_t lbeg = step1 ? 0 : L.step_off_cur;
-      if (threadIdx.x == 0) sh_snap[3] = step1 ? __ldcg(&c->touched_cnt) : __ldcg(&c->settled_cnt);
-      __syncthreads();
-      const uint32_t lend = (uint32_t)sh_snap[3];
+      const uint32_t lend = (uint32_t)sh_snap[3];  // (read behind the last round's barrier)
       const bool has = lbeg + qb * blockDim.x < lend;  // this block has settled vertices to count
       const int64_t wlo = L.ub - (int64_t)A.G.maxw > L.lb ? L.ub - (int64_t)A.G.maxw : L.lb;
-      const bool ring_sh = A.ring_shift == 0 && L.ub < EIC_INF_T && (L.ub - wlo) <= kShRing;
+      // The ring's first slots are counted in shared memory when a block settles at least as many vertices as that
+      // has slots (else clearing and flushing them costs more than the vertices' own atomics: 2 us a step on a
+      // grid). Distances beyond them go to the ring at once: in a window of 65535 most vertices share the first
+      // hundreds of slots, and a step of 2 M vertices took 288 us on those slots' atomics.
+      const uint32_t nset = lend - lbeg, per_block = max(min(nset, blockDim.x), nset / A.nb);
+      const uint32_t wslots = A.ring_shift == 0 && L.ub < EIC_INF_T ? (uint32_t)min((int64_t)kShRing, L.ub - wlo) : 0u;
+      const bool ring_sh = wslots && wslots <= per_block;
       const bool ring_narrow = ring_sh && (L.ub - wlo) <= kRingNarrow && A.G.max_deg < (1u << 27);  // (in shared memory)
+      const uint32_t ranks = min(A.G.D, (uint32_t)kShRanks);
       if (has) {
-        for (int r = threadIdx.x; r < kShRanks; r += blockDim.x) S.hist[r] = 0;
+        for (uint32_t r = threadIdx.x; r < ranks; r += blockDim.x) S.hist[r] = 0;
         if (ring_sh)
-          for (int r = threadIdx.x; r < kShRing; r += blockDim.x) S.ring[r] = 0;
+          for (uint32_t r = threadIdx.x; r < wslots; r += blockDim.x) S.ring[r] = 0;
+        if (threadIdx.x < 2) sh_red2[threadIdx.x] = 0;
       }
       __syncthreads();
-      unsigned long long bdeg = 0;
-      uint32_t bmax = 0, bany = 0;
+      uint32_t bdeg = 0, bmax1 = 0;  // degree sum (at most 2m < 2^32), 1 + the largest distance (0: none)
       const uint32_t nthreads = A.nb * blockDim.x;
       uint32_t xnext = 0;  // the single-query shape loads the next list entry one iteration ahead
       if constexpr (kRelaxIlp >= 2) {
@@ -1647,8 +1795,7 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
             __stcg(&A.scur[idx], cx);
           }
           bdeg += dg;
-          bmax = d > bmax ? d : bmax;
-          bany = 1;
+          bmax1 = max(bmax1, d + 1);
         }
         // degree histogram (internal vertices all have degree >= 1)
         if (!take) r = EIC_INF;
@@ -1660,52 +1807,46 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
         // distances; then one atomic per distinct slot in the warp, with the
         // group's degree sum (32-bit while 32 degrees cannot overflow it)
         const bool rk = take && (int64_t)d >= wlo && A.ring_shift == 0;  // (wide weights: Function 2 sums exactly)
-        const uint32_t slot = rk ? (ring_sh ? (uint32_t)(d - wlo) : (uint32_t)(((uint64_t)d >> A.ring_shift) & A.ring_mask))
-                                 : EIC_INF;
+        const uint32_t slot = rk ? (uint32_t)(d - wlo) : EIC_INF;
         if (ring_narrow) {
           const uint32_t rg = __match_any_sync(EIC_FULL_MASK, slot);
           const uint32_t sum = __reduce_add_sync(rg, rk ? dg : 0u);
-          if (rk && lane_id() == (uint32_t)__ffs(rg) - 1) atomicAdd(&S.ring[slot], (unsigned long long)sum);
+          if (rk && lane_id() == (uint32_t)__ffs(rg) - 1) atomicAdd(&S.ring[slot], sum);
         } else if (rk) {
-          if (ring_sh)
-            atomicAdd(&S.ring[slot], (unsigned long long)dg);
+          if (ring_sh && slot < wslots)
+            atomicAdd(&S.ring[slot], dg);
           else
-            atomicAdd(&A.ring[slot], (unsigned long long)dg);
+            atomicAdd(&A.ring[d & A.ring_mask], dg);
+        }
+      }
+      if (has) {  // block totals: one atomic each
+        bdeg = __reduce_add_sync(EIC_FULL_MASK, bdeg);
+        bmax1 = __reduce_max_sync(EIC_FULL_MASK, bmax1);
+        if (lane_id() == 0 && bmax1) {
+          atomicAdd(&sh_red2[0], bdeg);
+          atomicMax(&sh_red2[1], bmax1);
         }
       }
       __syncthreads();
       if (has) {
-        for (int r = threadIdx.x; r < kShRanks; r += blockDim.x)
+        for (uint32_t r = threadIdx.x; r < ranks; r += blockDim.x)
           if (S.hist[r]) atomicSub(&A.hist[r], S.hist[r]);
-        if (ring_sh)
-          for (int r = threadIdx.x; r < kShRing && r < L.ub - wlo; r += blockDim.x)
-            if (S.ring[r]) atomicAdd(&A.ring[((uint64_t)(wlo + r)) & A.ring_mask], S.ring[r]);
-      }
-      // block totals: degree sum and 1 + the largest distance (0: none), one atomic each
-      unsigned long long v[2] = {bdeg, bany ? (unsigned long long)bmax + 1 : 0ull};
-      v[0] = warp_sum_u64(v[0]);
-      for (int o = 16; o > 0; o >>= 1) v[1] = max(v[1], __shfl_xor_sync(EIC_FULL_MASK, v[1], o));
-      if ((threadIdx.x & 31) == 0) {
-        sh_red[threadIdx.x >> 5][0] = v[0];
-        sh_red[threadIdx.x >> 5][1] = v[1];
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        for (uint32_t w = 1; w < (blockDim.x >> 5); ++w) {
-          v[0] += sh_red[w][0];
-          v[1] = max(v[1], sh_red[w][1]);
+        for (uint32_t r = threadIdx.x; ring_sh && r < wslots; r += blockDim.x)
+          if (S.ring[r]) atomicAdd(&A.ring[(uint32_t)(wlo + r) & A.ring_mask], S.ring[r]);
+        if (threadIdx.x == 0 && sh_red2[1]) {
+          atomicAdd(&c->acc_deg, (unsigned long long)sh_red2[0]);
+          atomicMax(&c->acc_maxd1, sh_red2[1]);
         }
-        if (v[0]) atomicAdd(&c->acc_deg, v[0]);
-        if (v[1]) atomicMax(&c->acc_maxd1, (uint32_t)v[1]);
-        atom_add_acq_rel_u32(&c->s2_done, 1u);  // releases the block's statistics
+        __syncthreads();
       }
+      if (threadIdx.x == 0) red_release_add_u32(&c->s2_done, 1u);  // releases the block's statistics
       if (qb == 0) {  // block 0 waits (bounded) for every block's statistics
         if (threadIdx.x == 0) {
           uint64_t spins = 0;
           sh_last = 1;
           while (ld_acquire_u32(&c->s2_done) < A.nb) {
-            if (ld_volatile_int(&c->status) != 0 || ++spins > A.max_spin) {
-              atomicCAS(&c->status, 0, EIC_ETIMEOUT);
+            if (++spins > A.max_spin || ((spins & 15) == 0 && ld_volatile_int(&c->status) != 0)) {
+              barrier_fail(&c->bar, &c->status);
               sh_last = 0;
               break;
             }
@@ -1713,11 +1854,11 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, Gen& gen) {
           tl_mark(A, 4, L.rid);
         }
         __syncthreads();
-        if (sh_last) step_boundary<(kRelaxIlp >= 2), kFuse == 1>(A, P, B, L, rin);  // (the single-query shape inlines)
+        if (sh_last) step_boundary<(kRelaxIlp >= 2)>(A, P, B, L, rin);  // (the single-query shape inlines)
         if (threadIdx.x == 0) tl_mark(A, 5, L.rid);
       }
     }
-    if (!grid_barrier(&c->bar, &gen, A.nb, A.max_spin, &c->status)) break;
+    if (!grid_barrier(&c->bar, &ticket, A.nb, A.max_spin, &c->status)) break;
     if (qb == 0 && threadIdx.x == 0) tl_mark(A, 3, L.rid);
     read_ctl(c, L);
     if (L.done) break;
@@ -1787,12 +1928,10 @@ __device__ void ctl_init(const KArgs& A) {
   c->rounds_in_step = 0;
   c->trace_len = 0;
   c->tl_len = 0;
-  c->qcnt[0] = c->qcnt[1] = c->qcnt[2] = 0;
-  c->work[0] = c->work[1] = c->work[2] = 0;
+  c->rcnt[0] = c->rcnt[1] = c->rcnt[2] = make_uint2(0u, 0u);
   c->settled_cnt = 0;
   c->touched_cnt = 1;
   c->ub_cand = (G.highd0 > 0 && dgs >= G.highd0) ? 0u : EIC_INF;
-  c->tcnt[0] = c->tcnt[1] = c->tcnt[2] = 0;
   c->s2_done = 0;
   c->acc_maxd1 = 0;
   c->acc_deg = 0;
@@ -1803,10 +1942,10 @@ __device__ void ctl_init(const KArgs& A) {
 __global__ void k_init(KArgs A) {
   const DevGraph& G = A.G;
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < G.D; r += gridDim.x * blockDim.x) A.hist[r] = G.dcnt0[r];
-  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r <= A.ring_mask; r += gridDim.x * blockDim.x) A.ring[r] = 0;
+  if (A.ring_shift == 0)  // (wide weights: Function 2 clears the bins it uses)
+    for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r <= A.ring_mask; r += gridDim.x * blockDim.x) A.ring[r] = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl_init(A);
-    A.ctl->bar.count = 0;
     A.ctl->bar.arrived = 0;
     A.ctl->status = 0;
   }
@@ -1877,17 +2016,18 @@ struct BatchArgs {
 
 // The query's scratch at its starting values (what the single-query path
 // does with memsets and k_init), by the group's blocks.
-__device__ bool query_setup(const KArgs& A, uint32_t& gen) {
+__device__ bool query_setup(const KArgs& A, unsigned long long& ticket) {
   const DevGraph& G = A.G;
   const uint32_t stride = A.nb * blockDim.x, t0 = qblock(A) * blockDim.x + threadIdx.x;
   for (uint32_t i = t0; i < G.ni; i += stride) __stcg(&A.dist[i], EIC_INF);
   for (uint32_t i = t0; i < 2 * A.fwords; i += stride) __stcg(&A.fbits[i], 0u);
   for (uint32_t i = t0; i < A.fwords; i += stride) __stcg(&A.sbits[i], 0u);
   for (uint32_t r = t0; r < G.D; r += stride) __stcg(&A.hist[r], __ldg(&G.dcnt0[r]));
-  for (uint32_t r = t0; r <= A.ring_mask; r += stride) __stcg(&A.ring[r], 0ull);
-  if (!grid_barrier(&A.ctl->bar, &gen, A.nb, A.max_spin, &A.ctl->status)) return false;
+  if (A.ring_shift == 0)
+    for (uint32_t r = t0; r <= A.ring_mask; r += stride) __stcg(&A.ring[r], 0u);
+  if (!grid_barrier(&A.ctl->bar, &ticket, A.nb, A.max_spin, &A.ctl->status)) return false;
   if (qblock(A) == 0 && threadIdx.x == 0) ctl_init(A);
-  return grid_barrier(&A.ctl->bar, &gen, A.nb, A.max_spin, &A.ctl->status);
+  return grid_barrier(&A.ctl->bar, &ticket, A.nb, A.max_spin, &A.ctl->status);
 }
 
 // Distances in the caller's numbering (as k_output), by the group's blocks.
@@ -1912,11 +2052,11 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_batch(BatchArgs P) {
   const uint32_t grp = blockIdx.x / P.nb, qb = blockIdx.x % P.nb;
   const BatchSlot& W = P.slot[grp];
   Ctl* c = W.ctl;
-  uint32_t gen = __ldcg(&c->bar.gen);
+  unsigned long long ticket = 0;  // (the launch's preparation zeroed the arrival count)
   uint32_t qi = 0xFFFFFFFFu;
   for (;;) {
     if (qb == 0 && threadIdx.x == 0) c->next_q = ld_volatile_int(&c->status) == 0 ? atomicAdd(P.queue, 1u) : P.nq;
-    if (!grid_barrier(&c->bar, &gen, P.nb, P.max_spin, &c->status)) break;
+    if (!grid_barrier(&c->bar, &ticket, P.nb, P.max_spin, &c->status)) break;
     if (threadIdx.x == 0) sh_qi = __ldcg(&c->next_q);
     __syncthreads();
     qi = sh_qi;
@@ -1963,8 +2103,8 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_batch(BatchArgs P) {
       sA.fuse = bq.fuse;
     }
     __syncthreads();
-    if (!query_setup(sA, gen)) break;
-    run_query<kPullFastGroup, kRelaxIlpGroup, 2>(sA, Q, gen);
+    if (!query_setup(sA, ticket)) break;
+    run_query<kPullFastGroup, kRelaxIlpGroup, 2>(sA, Q, ticket);
     __syncthreads();
     if (ld_volatile_int(&c->status) != 0) break;
     query_output(sA);
@@ -1981,7 +2121,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_batch(BatchArgs P) {
 __global__ void k_batch_prep(BatchArgs P, uint32_t groups) {
   const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g < groups) {
-    P.slot[g].ctl->bar.count = 0;
+    P.slot[g].ctl->bar.arrived = 0;
     P.slot[g].ctl->status = 0;
   }
   if (g < P.nq) P.status[g] = EIC_EABORT;
@@ -2045,7 +2185,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_serve(ServeArgs P) {
   unsigned long long* finished = &P.claim[1];
   unsigned long long* idle_groups = &P.claim[2];
   unsigned long long* leave = &P.claim[3];
-  uint32_t gen = __ldcg(&c->bar.gen);
+  unsigned long long ticket = 0;  // (the launch's preparation zeroed the arrival count)
   unsigned long long mine = kNoTicket;  // first thread: the request it claimed last
   bool reported = true;                 // first thread: that request's completion is published
   bool registered = false;              // first thread: this group counts as idle
@@ -2095,7 +2235,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_serve(ServeArgs P) {
         reported = false;
       }
     }
-    if (!grid_barrier(&c->bar, &gen, P.nb, P.max_spin, &c->status)) break;
+    if (!grid_barrier(&c->bar, &ticket, P.nb, P.max_spin, &c->status)) break;
     if (threadIdx.x == 0) sh_t = __ldcg(&c->next_ticket);
     __syncthreads();
     const unsigned long long t = sh_t;
@@ -2148,13 +2288,13 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_serve(ServeArgs P) {
       sA.fuse = bq.fuse;
     }
     __syncthreads();
-    if (!query_setup(sA, gen)) break;
-    run_query<kPullFastGroup, kRelaxIlpGroup, 2>(sA, Q, gen);
+    if (!query_setup(sA, ticket)) break;
+    run_query<kPullFastGroup, kRelaxIlpGroup, 2>(sA, Q, ticket);
     __syncthreads();
     if (ld_volatile_int(&c->status) != 0) break;
     query_output(sA);
     // every block's part of the result is written before the group reports
-    if (!grid_barrier(&c->bar, &gen, P.nb, P.max_spin, &c->status)) break;
+    if (!grid_barrier(&c->bar, &ticket, P.nb, P.max_spin, &c->status)) break;
     if (qb == 0 && threadIdx.x == 0) {
       __threadfence_system();
       P.done[e].status = EIC_OK;
@@ -2182,7 +2322,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_serve(ServeArgs P) {
 __global__ void k_serve_prep(const BatchSlot* slot, uint32_t groups, unsigned long long* claim) {
   const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g < groups) {
-    slot[g].ctl->bar.count = 0;
+    slot[g].ctl->bar.arrived = 0;
     slot[g].ctl->status = 0;
   }
   if (g == 0) {
@@ -3073,12 +3213,12 @@ constexpr uint64_t kNaTouched = kNaScur + na_align((kNaN + 2) * 4);
 constexpr uint64_t kNaSbits = kNaTouched + na_align((kNaN + 1) * 4);
 constexpr uint64_t kNaHist = kNaSbits + na_align((kNaN / 32 + 2) * 4);
 constexpr uint64_t kNaRing = kNaHist + na_align(kNaD * 4);
-constexpr uint64_t kNaTaskOff = kNaRing + na_align((1ull << kNaRingBits) * 8);
+constexpr uint64_t kNaTaskOff = kNaRing + na_align((1ull << kNaRingBits) * 4);
 constexpr uint64_t kNaStepUb = kNaTaskOff + na_align(kNaTasks * sizeof(Task));
 constexpr uint64_t kNaStepOff = kNaStepUb + na_align((kNaS + 2) * 8);
 constexpr uint64_t kNaCtl = kNaStepOff + na_align((kNaS + 2) * 4);
 constexpr uint64_t kNaBytes = kNaCtl + na_align(sizeof(Ctl));
-static_assert(kNaBytes > 13000000 && kNaBytes < 14000000, "the header states the scratch size as about 13.4 MB");
+static_assert(kNaBytes > 13100000 && kNaBytes < 13250000, "the header states the scratch size as about 13.1 MB");
 
 static __device__ __align__(256) unsigned char g_na_scratch[kNaBytes];
 
@@ -3150,7 +3290,7 @@ extern "C" int eic_sssp_noalloc(const eic_graph* gc, uint32_t source, uint32_t* 
   A.touched = (uint32_t*)(b + kNaTouched);
   A.sbits = (uint32_t*)(b + kNaSbits);
   A.hist = (uint32_t*)(b + kNaHist);
-  A.ring = (unsigned long long*)(b + kNaRing);
+  A.ring = (uint32_t*)(b + kNaRing);
   A.tasks = (Task*)(b + kNaTaskOff);
   A.step_ub = (int64_t*)(b + kNaStepUb);
   A.step_off = (uint32_t*)(b + kNaStepOff);
