@@ -760,7 +760,7 @@ def main():
                          "frac": achieved / peak,
                          "traffic": None if args.road else MEASURED_TRAFFIC.get((args.scale, kernel_sources_sha256())),
                          "peak_kind": peak_kind,
-                         "kernel": ("k_eic_fused" if args.road else "k_eic") +
+                         "kernel": "k_eic"
                                    " (one launch per query; CUDA events around its launch)",
                          "kernel_ms_mean": statistics.mean(k_ms), "alg_bytes_mean": statistics.mean(b_alg)},
             "cpu_baseline": cpu, "clocks": clocks, "e2e": e2e, "gpu_launches": 3 * q * args.steps,

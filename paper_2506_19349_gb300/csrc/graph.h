@@ -36,7 +36,7 @@ struct Ctl {
   uint32_t trace_len;
   uint32_t tl_len;  // diagnostic timeline events recorded
   // appended with atomics during phases
-  uint2 rcnt[3];  // by round id mod 3: vertices queued for the next round, tasks of the round
+  uint4 rcnt[3];  // by round id mod 3: vertices queued for the next round, tasks of the round, 1: the next round is plain
   uint32_t settled_cnt;
   uint32_t touched_cnt;
   uint32_t ub_cand;
@@ -58,13 +58,18 @@ struct BatchQuery {
   uint32_t s;
   uint32_t ring_mask, ring_shift, task_cap;
   uint32_t gap_shift, heavy_min;  // step-width scaling and window-class threshold for this query's graph
-  uint32_t fuse;                  // 1: fused rounds (every degree of the graph <= heavy_min)
+  uint32_t fuse;                  // rounds of at most this many items per warp are fused (fuse_items)
 };
 
-// Fused rounds (bucket fusion) apply to a graph whose every degree is at most
-// heavy_min (no window becomes a grid task), unless the caller turns them off.
-inline bool fuse_ok(const DevGraph& G, uint32_t heavy_min, uint32_t flags) {
-  return G.max_deg <= heavy_min && !(flags & EIC_FLAG_NO_FUSE);
+// Fused rounds (bucket fusion): the items per warp up to which a round is
+// fused, 0 when the caller turns them off. Graphs whose every degree is at
+// most heavy_min (road-like: many rounds of short windows) fuse whatever the
+// warps can take at once; others their small rounds (RMAT 131 k: 543, 527 us
+// at 4 and 16 items a warp, 579 without).
+constexpr uint32_t kFuseRoad = 32, kFuseItems = 16;
+inline uint32_t fuse_items(const DevGraph& G, uint32_t heavy_min, uint32_t flags) {
+  if (flags & EIC_FLAG_NO_FUSE) return 0;
+  return G.max_deg <= heavy_min ? kFuseRoad : kFuseItems;
 }
 
 // Scratch of one block group, reused by every query the group runs.
@@ -112,7 +117,6 @@ struct Workspace {
   uint32_t task_cap = 0, step_cap = 0;
   uint64_t bytes = 0;
   int grid = 0, block = 0;  // cached cooperative launch shape of k_eic
-  int grid_fused = 0, block_fused = 0;  // and of k_eic_fused
 };
 
 struct eic_graph {

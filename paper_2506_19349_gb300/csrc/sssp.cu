@@ -92,7 +92,7 @@ struct KArgs {
   unsigned long long* timeline;  // NULL unless the caller asked for it
   uint32_t timeline_cap;
   uint32_t nb;  // blocks working on this query: the grid, or one block group of a batch
-  uint32_t fuse;  // fused rounds for this query (kernels that decide per query)
+  uint32_t fuse;  // rounds of at most this many items per warp are fused (see fuse_items; 0: none)
 };
 
 // Index of the block within the blocks that work on its query.
@@ -134,6 +134,12 @@ struct RoundScr {
 // and 123, 117, 119 and 121 ms on a 4096^2 grid (short ones: less to wait for).
 constexpr uint32_t kFuseWarps = 8;
 constexpr uint32_t kFusePop = 8;      // queued vertices a warp takes at a time
+// Graphs with long rows: the longest window of a wave, and the 32-entry
+// iterations after which a warp's group hands on what is left. RMAT 250 k with
+// wide weights, 1.48 ms without fused rounds: 1.41, 1.47 and 1.50 ms at 6, 16
+// and 32 iterations; windows of 64 and 256 entries differ by 2% either way.
+constexpr uint32_t kFuseLong = 64;
+constexpr uint32_t kFuseIters = 6;
 constexpr uint32_t kFuseQueue = 128 * kFuseWarps;  // entries of a local queue (a power of two)
 constexpr uint32_t kFuseGroups = (kMaxWarps + kFuseWarps - 1) / kFuseWarps;
 static_assert(kFuseGroups <= 15, "a group synchronises on named barrier 1 + its index; 0 is the block barrier");
@@ -146,7 +152,7 @@ struct Stage {
     };
     uint4 fq[kFuseGroups][kFuseQueue];  // {vertex, distance, row begin, degree}
   };
-  uint32_t fcnt[kFuseGroups][3];  // entries pushed to the local queue, by wave mod 3
+  uint32_t fcnt[kFuseGroups][4];  // entries pushed to the local queue, by wave mod 3
   uint32_t wf[kMaxWarps][kWarpStage];
 };
 
@@ -358,6 +364,7 @@ struct RoundCtx {
   uint32_t* first_list;
   uint32_t* first_cnt;
   uint32_t* tcnt;
+  uint32_t* plain_out;  // set: the next round must be a plain one
 };
 
 // Flush the block's task stage to the global list (block-uniform call).
@@ -985,10 +992,9 @@ __device__ __noinline__ int64_t block_st_exact_call(const KArgs& A, S3Scr& S, in
   return block_st_exact(A, S, ub, sumd_ub, gap_lb, gap_ub_raw, y, st0, st1, j0, step, send);
 }
 
-// A fused round: the FUSED local iterations of Section 4.1 (bucket fusion),
-// for graphs in which no window is longer than heavy_min (every degree <=
-// heavy_min, so there are no grid tasks), in every round of a step after the
-// first (and its first round too when the step has no pull). The round's
+// A fused round: the FUSED local iterations of Section 4.1 (bucket fusion), in
+// a step's rounds after the first (and its first round too when the step has
+// no pull) that have few enough items (fuse_items). The round's
 // frontier vertices (or the push set, whose windows start at their cursors)
 // are dealt evenly to groups of kFuseWarps warps all over the query's blocks.
 // A group relaxes its vertices' windows; every vertex it improves goes into
@@ -1010,6 +1016,17 @@ __device__ __noinline__ int64_t block_st_exact_call(const KArgs& A, S3Scr& S, in
 // row bounds, entries, distance, atomicMin): a round of the 4096^2 grid went
 // from 26.1 to 14.4 us, its query from 168 to 118 ms, and the 1531 x 977 grid
 // at gap_shift 4 from 18.7 to 7.2 ms.
+//
+// kRoad: no window is longer than heavy_min (every degree of the graph is at
+// most that). Otherwise a window may be too long for one warp: an item's then
+// becomes grid tasks, a vertex improved in the round waits for the next, plain
+// round; and a group that has spent kFuseIters iterations hands its queue to
+// the next round, where it is dealt to all warps again (34 items whose subtree
+// of 5000 vertices stayed in 34 groups took 220 us, plain rounds 130 us). On
+// such graphs it saves the 8 us of each small round: uniform 2^14 vertices 488
+// -> 394 us, RMAT 131 k 579 -> 518 us, RMAT 2^22 1029 -> 990 us, RMAT 2^25
+// 3.03 -> 2.94 ms a query.
+template <bool kRoad>
 __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, RoundScr& S, Stage& T,
                             uint32_t nitems, bool round1, const uint32_t* qin, Counters& C) {
   const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
@@ -1027,13 +1044,15 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
   uint32_t i0 = min(nitems, (grp * A.nb + qblock(A)) * per);
   const uint32_t i1 = min(nitems, i0 + per);
   const uint32_t np = round1 ? L.push_end - L.push_beg : 0;
-  if (gw == 0 && lane < 3) fcnt[lane] = 0;
+  if (gw == 0 && lane < 4) fcnt[lane] = 0;
   group_sync();
+  uint32_t spent = 0;
   uint32_t lh = 0, lt = 0, wave = 0;  // the ring's head and tail, the wave mod 3 (the same in every thread of the group)
   while (i0 < i1 || lh != lt) {
     uint32_t d = EIC_INF, b = 0, len = 0, u = 0, rb = 0, deg = 0;
     uint32_t now = EIC_INF;  // a queued vertex's distance as its wave begins
     bool vertex = false;     // a frontier vertex (or the source): its window starts at its row
+    bool seed = false;       // one of the round's items
     const uint32_t room = kFuseQueue - (lt - lh);
     if (i0 < i1) {
       const uint32_t take = min(i1 - i0, 32 * gn), each = (take + gn - 1) / gn;
@@ -1059,6 +1078,7 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
           }
           now = d;
         }
+        seed = true;
       } else if (mine) {  // a frontier vertex, or in a step's first round the source, once
         u = round1 ? L.s_int : ld_list(&qin[i]);
         const uint2 rr = row_of(A.G, u);
@@ -1066,6 +1086,7 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
         deg = rr.y;
         d = now = __ldcg(&A.dist[u]);
         vertex = d != EIC_INF && !(d > 0 && deg == 1);  // Paths excludes leaves (Algorithm 1)
+        seed = true;
       }
     } else {
       const uint32_t take = min(lt - lh, kFusePop * gn), each = (take + gn - 1) / gn;
@@ -1089,8 +1110,36 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
       if (deg > kCursorMin) {
         const uint32_t e = gallop_w(A.G.adj, rb, rb + deg, R.ub_eff - (int64_t)d);
         __stcg(&A.cursor[u], e - rb);
-        len = e - rb;
+        if ((int64_t)d < R.lb) b = lower_bound_w(A.G.adj, rb, e, R.lb - (int64_t)d);  // (the source)
+        len = e - b;
       }
+    }
+    if (!kRoad && __any_sync(EIC_FULL_MASK, len > kFuseLong)) {
+      // Windows too long for a wave. An item's becomes grid tasks, once per
+      // vertex and round (what the task list is sized for); a vertex improved
+      // in this round goes to the next one, which is then a plain round.
+      const bool lng = len > kFuseLong;
+      uint32_t emit = __ballot_sync(EIC_FULL_MASK, lng && seed);
+      while (emit) {
+        const int src = __ffs(emit) - 1;
+        emit &= emit - 1;
+        const uint32_t tb = __shfl_sync(EIC_FULL_MASK, b, src), tl = __shfl_sync(EIC_FULL_MASK, len, src);
+        const uint32_t tu = __shfl_sync(EIC_FULL_MASK, u, src), td = __shfl_sync(EIC_FULL_MASK, d, src);
+        const uint32_t ntask = (tl + kTaskLen - 1) / kTaskLen;
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(R.tcnt, ntask);
+        at = __shfl_sync(EIC_FULL_MASK, at, 0);
+        for (uint32_t k = lane; k < ntask; k += 32)
+          A.tasks[at + k] = Task{tb + k * kTaskLen, min(kTaskLen, tl - k * kTaskLen), tu, td};
+        if (lane == 0) C.heavy += ntask;
+      }
+      const bool sap = lng && !seed && claim_bit(R, u);
+      const uint32_t slot = warp_append(sap, R.qcnt_out);
+      if (sap) {
+        __stcg(&R.qout[slot], u);
+        __stcg(R.plain_out, 1u);
+      }
+      if (lng) len = 0;
     }
     const uint32_t incl = warp_incl_scan(len);
     const uint32_t total = __shfl_sync(EIC_FULL_MASK, incl, 31);
@@ -1099,6 +1148,10 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
     W.val[lane] = d;
     __syncwarp();
     uint32_t live = 0;  // lanes whose vertex still has the distance it was queued with
+    if (!kRoad) {
+      spent += (total + 31) / 32;
+      if (spent > kFuseIters && lane == 0) fcnt[3] = 1;
+    }
     for (uint32_t g0 = 0; g0 < total; g0 += 32) {
       const uint32_t g = g0 + lane;
       uint32_t own = 0;
@@ -1157,6 +1210,16 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
     lt += min(fcnt[wave], room);
     if (gw == 0 && lane == 0) fcnt[wave == 0 ? 2 : wave - 1] = 0;  // read by all before this barrier, next used two waves on
     wave = wave == 2 ? 0 : wave + 1;
+    if (!kRoad && fcnt[3] && i0 >= i1) {  // long enough alone: the rest goes to the next round
+      for (uint32_t i = lh + gw * 32; i < lt; i += gn * 32) {
+        const bool in = i + lane < lt;
+        const uint32_t v = in ? fq[(i + lane) & (kFuseQueue - 1)].x : 0u;
+        const bool sap = in && claim_bit(R, v);
+        const uint32_t slot = warp_append(sap, R.qcnt_out);
+        if (sap) __stcg(&R.qout[slot], v);
+      }
+      break;
+    }
   }
   warp_flush(Fw);
   tl_block(A, 6, R.rid);
@@ -1604,8 +1667,7 @@ struct QueryShared {
 // The query loop of Algorithm 1 run by the A.nb blocks of one query: rounds
 // of a step (item phase, task phase), statistics pass, step boundary, until
 // termination. ticket is the block's arrival ticket of the query's barrier.
-// kFuse: 0 no fused rounds, 1 fused rounds, 2 as A.fuse says (per query).
-template <uint32_t kPullFast, uint32_t kRelaxIlp, uint32_t kFuse = 0>
+template <uint32_t kPullFast, uint32_t kRelaxIlp>
 __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ticket) {
   PhaseScr& P = Q.P;
   Stage& T = Q.T;
@@ -1642,6 +1704,7 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ti
   while (alive) {
     // ------------------------------------------------ rounds of one step
     uint32_t rin = 0;
+    bool plain = false;  // the round must be a plain one
     for (;;) {
       ++L.rid;
       if (++total_rounds > kMaxRounds) {
@@ -1652,7 +1715,7 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ti
       const bool round1 = (L.step >= 2 && rin == 0);
       // counters of round rid+1 were last read two barriers ago: clear them now
       if (qb == 0 && threadIdx.x == 0) {
-        __stcg(&c->rcnt[(L.rid + 1) % 3], make_uint2(0u, 0u));
+        __stcg(&c->rcnt[(L.rid + 1) % 3], make_uint4(0u, 0u, 0u, 0u));
       }
       if (L.cur_cnt) {  // the other bitmap served round rid-1 (which set a bit per vertex it queued) and is
                         // next used in round rid+1: clear it now
@@ -1674,36 +1737,41 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ti
       R.first_list = R.step1 ? A.touched : A.sid;
       R.first_cnt = R.step1 ? &c->touched_cnt : &c->settled_cnt;
       R.tcnt = &c->rcnt[L.rid % 3].y;
+      R.plain_out = &c->rcnt[L.rid % 3].z;
       const uint32_t* qin = L.qsel ? A.q1 : A.q0;
       Local LL = L;
       if (!L.pull_on) LL.pull_cnt = 0;
       const uint32_t nitems = round1 ? (LL.push_end - LL.push_beg) + LL.pull_cnt + LL.extra_s : L.cur_cnt;
       if (qb == 0 && threadIdx.x == 0) tl_mark(A, 8, nitems);  // diagnostic: the round's items
-      if ((kFuse == 1 || (kFuse == 2 && A.fuse)) && !R.step1 && (!round1 || !LL.pull_on) &&
-          nitems <= 32u * A.nb * (blockDim.x >> 5))
-        fused_round(A, R, LL, P.r, T, nitems, round1, qin, C);
-      else
+      if (!R.step1 && (!round1 || !LL.pull_on) && !plain && nitems <= A.fuse * A.nb * (blockDim.x >> 5)) {
+        if (A.fuse == kFuseRoad)
+          fused_round<true>(A, R, LL, P.r, T, nitems, round1, qin, C);
+        else
+          fused_round<false>(A, R, LL, P.r, T, nitems, round1, qin, C);
+      } else {
         round_phase<kPullFast, kRelaxIlp>(A, R, LL, P.r, T, nitems, round1, qin, C);
+      }
       if (!grid_barrier(&c->bar, &ticket, A.nb, A.max_spin, &c->status)) {
         alive = false;
         break;
       }
       if (threadIdx.x == 0) {
-        const uint2 rc = __ldcg(&c->rcnt[L.rid % 3]);
-        sh_snap[0] = rc.y;
+        const uint4 rc = __ldcg(&c->rcnt[L.rid % 3]);
+        sh_snap[0] = rc.y | (unsigned long long)rc.z << 32;
         sh_snap[1] = rc.x;
         sh_snap[2] = __ldcg(&c->ub_cand);
         sh_snap[3] = __ldcg(R.first_cnt);
         if (qb == 0) tl_mark(A, 1, L.rid);
       }
       __syncthreads();
-      const unsigned long long hp = sh_snap[0];
+      const uint32_t hp = (uint32_t)sh_snap[0];
+      const bool plain_next = sh_snap[0] >> 32;
       L.cur_cnt = (uint32_t)sh_snap[1];
       uint32_t uc = (uint32_t)sh_snap[2];
       __syncthreads();
       if (hp != 0) {
-        if (qb == 0 && threadIdx.x == 0) tl_mark(A, 9, (uint32_t)hp);  // diagnostic: the round's tasks
-        task_phase<(kRelaxIlp >= 2)>(A, R, (uint32_t)hp, T, C);
+        if (qb == 0 && threadIdx.x == 0) tl_mark(A, 9, hp);  // diagnostic: the round's tasks
+        task_phase<(kRelaxIlp >= 2)>(A, R, hp, T, C);
         if (!grid_barrier(&c->bar, &ticket, A.nb, A.max_spin, &c->status)) {
           alive = false;
           break;
@@ -1721,6 +1789,7 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ti
       }
       if (R.step1 && uc != EIC_INF && (int64_t)uc < L.ub) L.ub = uc;
       L.qsel ^= 1u;
+      plain = plain_next;
       ++rin;
       if (L.cur_cnt == 0) break;
     }
@@ -1884,15 +1953,6 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic(KArgs A) {
   run_query<kPullFastSingle, kRelaxIlpSingle>(A, Q, ticket);
 }
 
-// The same query with fused rounds (bucket fusion), for graphs whose every
-// degree is at most heavy_min: road-like graphs, whose steps take many small
-// rounds.
-__global__ void __launch_bounds__(kMaxBlock, 2) k_eic_fused(KArgs A) {
-  __shared__ QueryShared Q;
-  unsigned long long ticket = 0;  // (k_init zeroed the arrival count)
-  run_query<kPullFastSingle, kRelaxIlpSingle, 1>(A, Q, ticket);
-}
-
 // Control block of a new query (one thread): the source's distance, the
 // first round's frontier {s}, step 1 = <0, +inf> with st = 0, and gap(0).
 __device__ void ctl_init(const KArgs& A) {
@@ -1928,7 +1988,7 @@ __device__ void ctl_init(const KArgs& A) {
   c->rounds_in_step = 0;
   c->trace_len = 0;
   c->tl_len = 0;
-  c->rcnt[0] = c->rcnt[1] = c->rcnt[2] = make_uint2(0u, 0u);
+  c->rcnt[0] = c->rcnt[1] = c->rcnt[2] = make_uint4(0u, 0u, 0u, 0u);
   c->settled_cnt = 0;
   c->touched_cnt = 1;
   c->ub_cand = (G.highd0 > 0 && dgs >= G.highd0) ? 0u : EIC_INF;
@@ -2104,7 +2164,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_batch(BatchArgs P) {
     }
     __syncthreads();
     if (!query_setup(sA, ticket)) break;
-    run_query<kPullFastGroup, kRelaxIlpGroup, 2>(sA, Q, ticket);
+    run_query<kPullFastGroup, kRelaxIlpGroup>(sA, Q, ticket);
     __syncthreads();
     if (ld_volatile_int(&c->status) != 0) break;
     query_output(sA);
@@ -2289,7 +2349,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_serve(ServeArgs P) {
     }
     __syncthreads();
     if (!query_setup(sA, ticket)) break;
-    run_query<kPullFastGroup, kRelaxIlpGroup, 2>(sA, Q, ticket);
+    run_query<kPullFastGroup, kRelaxIlpGroup>(sA, Q, ticket);
     __syncthreads();
     if (ld_volatile_int(&c->status) != 0) break;
     query_output(sA);
@@ -2387,27 +2447,21 @@ struct DeviceGuard {
   ~DeviceGuard() { cudaSetDevice(prev); }
 };
 
-// The cooperative grid of the query kernel (k_eic, or k_eic_fused), cached
-// per workspace for the block size last used.
-int launch_shape(Workspace* ws, int block, bool fused) {
-  int& grid = fused ? ws->grid_fused : ws->grid;
-  int& cached = fused ? ws->block_fused : ws->block;
-  if (grid && cached == block) return EIC_OK;
+// The cooperative grid of the query kernel, cached per workspace for the block
+// size last used.
+int launch_shape(Workspace* ws, int block) {
+  if (ws->grid && ws->block == block) return EIC_OK;
   int dev = 0, sms = 0, per_sm = 0, coop = 0;
   EIC_CUDA_TRY(cudaGetDevice(&dev));
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
   if (!coop) return EIC_ECUDA;
-  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused ? k_eic_fused : k_eic, block, 0));
+  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eic, block, 0));
   if (per_sm < 1) return EIC_ECUDA;
-  grid = sms * per_sm;
-  cached = block;
+  ws->grid = sms * per_sm;
+  ws->block = block;
   return EIC_OK;
 }
-
-// Fused rounds (bucket fusion) apply to graphs whose every degree is at most
-// heavy_min, unless the caller turns them off.
-bool use_fused(const eic_graph* g, const eic_params& p) { return fuse_ok(g->dg, p.heavy_min, p.flags); }
 
 KArgs make_args(eic_graph* g, uint32_t s, uint32_t* dist, const eic_params& p, int* status_out, int grid) {
   Workspace& w = g->ws;
@@ -2449,7 +2503,7 @@ KArgs make_args(eic_graph* g, uint32_t s, uint32_t* dist, const eic_params& p, i
   A.timeline = nullptr;
   A.timeline_cap = 0;
   A.nb = (uint32_t)grid;
-  A.fuse = 0;  // (the single-query kernels fix it: k_eic_fused or k_eic)
+  A.fuse = fuse_items(g->dg, p.heavy_min, p.flags);
   return A;
 }
 
@@ -2458,10 +2512,9 @@ int enqueue_query(eic_graph* g, uint32_t s, uint32_t* dist, uint32_t* parent, co
                   cudaStream_t st, bool timeline = false, cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr) {
   Workspace& w = g->ws;
   const int block = p.block_threads ? (int)p.block_threads : kDefaultBlock;
-  const bool fused = use_fused(g, p);
-  int rc = launch_shape(&w, block, fused);
+  int rc = launch_shape(&w, block);
   if (rc) return rc;
-  const int grid = fused ? w.grid_fused : w.grid;
+  const int grid = w.grid;
   EIC_CUDA_TRY(cudaMemsetAsync(w.idist, 0xFF, (uint64_t)g->dg.ni * 4, st));
   EIC_CUDA_TRY(cudaMemsetAsync(w.sbits, 0, ((uint64_t)g->dg.ni / 32 + 2) * 4, st));
   EIC_CUDA_TRY(cudaMemsetAsync(w.fbits, 0, 2 * ((uint64_t)g->dg.ni / 32 + 2) * 4, st));
@@ -2474,8 +2527,7 @@ int enqueue_query(eic_graph* g, uint32_t s, uint32_t* dist, uint32_t* parent, co
   EIC_CUDA_TRY(cudaGetLastError());
   void* args[] = {&A};
   if (ev0) EIC_CUDA_TRY(cudaEventRecord(ev0, st));
-  EIC_CUDA_TRY(cudaLaunchCooperativeKernel(fused ? (const void*)k_eic_fused : (const void*)k_eic, dim3(grid),
-                                           dim3(block), args, 0, st));
+  EIC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_eic, dim3(grid), dim3(block), args, 0, st));
   if (ev1) EIC_CUDA_TRY(cudaEventRecord(ev1, st));
   k_output<<<4 * grid, 256, 0, st>>>(g->dg, w.idist, s, dist);
   EIC_CUDA_TRY(cudaGetLastError());
@@ -2873,7 +2925,7 @@ int batch_create(const eic_graph* const* graphs, const uint32_t* sources, uint32
     q.task_cap = (uint32_t)(G.two_m / kHeavyMinFloor + 2);
     q.gap_shift = p.gap_shift;
     q.heavy_min = p.heavy_min;
-    q.fuse = fuse_ok(G, p.heavy_min, p.flags) ? 1u : 0u;
+    q.fuse = fuse_items(G, p.heavy_min, p.flags);
     b->hq.push_back(q);
     b->order.push_back(i);
     b->qgraph.push_back(graphs[i]);
@@ -3042,7 +3094,7 @@ int eic_batch_tune(eic_batch* b, void* stream, eic_batch_config* best) {
     auto trial = [&](uint32_t g, uint32_t block, uint32_t hm, double* ms_out) -> int {
       for (auto& q : b->hq) {
         q.heavy_min = hm;
-        q.fuse = fuse_ok(q.G, hm, b->p.flags) ? 1u : 0u;
+        q.fuse = fuse_items(q.G, hm, b->p.flags);
       }
       b->p.heavy_min = hm;
       int r = batch_upload(b);
@@ -3137,7 +3189,7 @@ int eic_batch_tune(eic_batch* b, void* stream, eic_batch_config* best) {
     // keep the winner; the scratch shrinks to its group count
     for (auto& q : b->hq) {
       q.heavy_min = best_hm;
-      q.fuse = fuse_ok(q.G, best_hm, b->p.flags) ? 1u : 0u;
+      q.fuse = fuse_items(q.G, best_hm, b->p.flags);
     }
     b->p.heavy_min = best_hm;
     if ((rc = batch_upload(b))) return rc;
@@ -3313,7 +3365,7 @@ extern "C" int eic_sssp_noalloc(const eic_graph* gc, uint32_t source, uint32_t* 
   A.timeline = nullptr;
   A.timeline_cap = 0;
   A.nb = (uint32_t)nd.grid;
-  A.fuse = 0;
+  A.fuse = fuse_items(G, A.heavy_min, A.flags);
   // Once anything is enqueued, every return waits for the stream first: the
   // next call may reuse the scratch only when this call's work has finished.
   auto enqueue = [&]() -> int {
