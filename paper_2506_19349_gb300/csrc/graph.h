@@ -94,6 +94,7 @@ struct BatchSlot {
 
 struct Workspace {
   uint32_t n = 0;
+  unsigned char* base = nullptr;  // the one allocation that holds the arrays
   uint32_t* idist = nullptr;  // distances in internal ids
   uint32_t* fbits = nullptr;  // two frontier-insertion bitmaps
   uint32_t* q[2] = {nullptr, nullptr};

@@ -2,6 +2,7 @@
 // of one group's arrays, and a pool of groups in one device allocation.
 #pragma once
 
+#include <mutex>
 #include <vector>
 
 #include "graph.h"
@@ -24,7 +25,7 @@ struct SlotLayout {
       ctl, bytes;
 };
 
-inline SlotLayout slot_layout(const SlotCaps& c) {
+inline SlotLayout slot_layout(const SlotCaps& c, uint64_t step_cap = kBatchStepCap) {
   SlotLayout L;
   uint64_t o = 0;
   auto take = [&o](uint64_t bytes) {
@@ -46,8 +47,8 @@ inline SlotLayout slot_layout(const SlotCaps& c) {
   L.hist = take(((uint64_t)c.D + 1) * 4);
   L.ring = take((1ull << c.ring_bits) * 4);
   L.tasks = take((c.two_m / kHeavyMinFloor + 2) * sizeof(Task));
-  L.step_ub = take(((uint64_t)kBatchStepCap + 2) * 8);
-  L.step_off = take(((uint64_t)kBatchStepCap + 2) * 4);
+  L.step_ub = take((step_cap + 2) * 8);
+  L.step_off = take((step_cap + 2) * 4);
   L.ctl = take(sizeof(Ctl));
   L.bytes = o;
   return L;
@@ -116,6 +117,38 @@ struct SlotPool {
     count = groups;
     slot_bytes = L.bytes;
     return EIC_OK;
+  }
+};
+
+// Pinned host mirrors of control blocks: 128 slots of one small allocation,
+// made at the first use and kept, since page-locking and unlocking a few
+// hundred bytes takes 0.3 ms a graph. get() gives nullptr when every slot is
+// taken; put() takes back a slot of this pool and says whether it was one.
+struct PinnedSlots {
+  static constexpr uint32_t kSlots = 128, kBytes = 512;
+  std::mutex mu;
+  unsigned char* base = nullptr;
+  uint64_t taken[kSlots / 64] = {};
+  void* get() {
+    std::lock_guard<std::mutex> lock(mu);
+    if (!base && cudaHostAlloc((void**)&base, kSlots * kBytes, cudaHostAllocPortable) != cudaSuccess) {
+      (void)cudaGetLastError();
+      base = nullptr;
+      return nullptr;
+    }
+    for (uint32_t k = 0; k < kSlots; ++k)
+      if (!(taken[k / 64] >> (k % 64) & 1)) {
+        taken[k / 64] |= 1ull << (k % 64);
+        return base + k * kBytes;
+      }
+    return nullptr;
+  }
+  bool put(void* p) {
+    std::lock_guard<std::mutex> lock(mu);
+    const uint64_t off = (uint64_t)((unsigned char*)p - base);
+    if (!base || (unsigned char*)p < base || off >= kSlots * kBytes) return false;
+    taken[off / kBytes / 64] &= ~(1ull << (off / kBytes % 64));
+    return true;
   }
 };
 

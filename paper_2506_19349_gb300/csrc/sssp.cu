@@ -2406,18 +2406,6 @@ constexpr int kDefaultBlock = 512;
 constexpr uint32_t kDefaultSpinLog2 = 22;
 constexpr uint32_t kStNumMax = 1u << 16;  // Function 2's candidate bins fit the 2^20-slot ring of wide weights
 
-template <typename T>
-int walloc(Workspace* ws, T** p, uint64_t count) {
-  *p = nullptr;
-  if (count == 0) count = 1;
-  if (cudaMalloc((void**)p, count * sizeof(T)) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return EIC_ENOMEM;
-  }
-  ws->bytes += count * sizeof(T);
-  return EIC_OK;
-}
-
 int resolve_params(const eic_params* in, eic_params* out) {
   if (in) {
     *out = *in;
@@ -2581,26 +2569,13 @@ int output_view(int dev, uint32_t* p, uint32_t** out) {
 
 }  // namespace
 
+namespace {
+PinnedSlots g_mirrors;
+}  // namespace
+
 void eic_ws_free(Workspace* w) {
-  cudaFree(w->idist);
-  cudaFree(w->fbits);
-  cudaFree(w->q[0]);
-  cudaFree(w->q[1]);
-  cudaFree(w->sid);
-  cudaFree(w->sd);
-  cudaFree(w->scur);
-  cudaFree(w->cursor);
-  cudaFree(w->touched);
-  cudaFree(w->sbits);
-  cudaFree(w->hist);
-  cudaFree(w->ring);
-  cudaFree(w->tasks);
-  cudaFree(w->step_ub);
-  cudaFree(w->step_off);
-  cudaFree(w->trace);
-  cudaFree(w->timeline);
-  cudaFree(w->ctl);
-  if (w->ctl_host) cudaFreeHost(w->ctl_host);
+  cudaFree(w->base);
+  if (w->ctl_host && !g_mirrors.put(w->ctl_host)) cudaFreeHost(w->ctl_host);
   if (w->ev[0]) cudaEventDestroy(w->ev[0]);
   if (w->ev[1]) cudaEventDestroy(w->ev[1]);
   *w = Workspace();
@@ -2610,29 +2585,48 @@ int eic_ws_ensure(eic_graph* g, int) {
   Workspace* w = &g->ws;
   if (w->ctl) return EIC_OK;
   const DevGraph& G = g->dg;
-  const uint64_t n = G.ni;  // per-vertex arrays cover the internal (non-isolated) vertices
-  int rc = EIC_OK;
-  uint32_t maxw = G.maxw ? G.maxw : 1;
-  uint32_t bits = 0;
-  while (bits < 32 && (1ull << bits) <= maxw) ++bits;  // 2^bits > maxW
-  w->ring_bits = bits < 20 ? bits : 20;
-  w->ring_shift = bits > 20 ? bits - 20 : 0;  // nonzero: Function 2 sums exactly, the ring holds its bins
+  w->ring_bits = ring_layout(G.maxw, &w->ring_shift);
   // a window longer than heavy_min >= 16 yields ceil(len / 64) <= len / 16 tasks,
   // and the windows of one round belong to distinct vertices
   w->task_cap = (uint32_t)(G.two_m / kHeavyMinFloor + 2);
   w->step_cap = kStepCap;
-  w->n = G.ni;
-  if ((rc = walloc(w, &w->idist, n)) || (rc = walloc(w, &w->fbits, 2 * (n / 32 + 2))) || (rc = walloc(w, &w->q[0], n)) || (rc = walloc(w, &w->q[1], n)) ||
-      (rc = walloc(w, &w->sid, n + 2)) || (rc = walloc(w, &w->sd, n + 2)) ||
-      (rc = walloc(w, &w->scur, n + 2)) || (rc = walloc(w, &w->cursor, n)) || (rc = walloc(w, &w->touched, n + 1)) || (rc = walloc(w, &w->sbits, n / 32 + 2)) ||
-      (rc = walloc(w, &w->hist, (uint64_t)G.D + 1)) || (rc = walloc(w, &w->ring, 1ull << w->ring_bits)) ||
-      (rc = walloc(w, &w->tasks, w->task_cap)) || (rc = walloc(w, &w->step_ub, (uint64_t)kStepCap + 2)) ||
-      (rc = walloc(w, &w->step_off, (uint64_t)kStepCap + 2)) || (rc = walloc(w, &w->trace, kTraceCap)) || (rc = walloc(w, &w->timeline, 2ull * kTimelineCap)) ||
-      (rc = walloc(w, &w->ctl, 1))) {
-    eic_ws_free(w);
-    return rc;
+  w->n = G.ni;  // per-vertex arrays cover the internal (non-isolated) vertices
+  SlotCaps caps;
+  caps.ni = G.ni;
+  caps.two_m = G.two_m;
+  caps.D = G.D;
+  caps.ring_bits = w->ring_bits;
+  const SlotLayout L = slot_layout(caps, kStepCap);  // one allocation: 19 of them took 0.5 ms, and freeing them as long
+  const uint64_t trace = L.bytes, timeline = trace + ((kTraceCap * sizeof(eic_step) + 255) & ~255ull);
+  const uint64_t bytes = timeline + 2ull * kTimelineCap * 8;
+  if (cudaMalloc((void**)&w->base, bytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    *w = Workspace();
+    return EIC_ENOMEM;
   }
-  if (cudaMallocHost((void**)&w->ctl_host, sizeof(Ctl)) != cudaSuccess) {
+  unsigned char* b = w->base;
+  w->bytes = bytes;
+  w->idist = (uint32_t*)(b + L.idist);
+  w->fbits = (uint32_t*)(b + L.fbits);
+  w->cursor = (uint32_t*)(b + L.cursor);
+  w->q[0] = (uint32_t*)(b + L.q0);
+  w->q[1] = (uint32_t*)(b + L.q1);
+  w->sid = (uint32_t*)(b + L.sid);
+  w->sd = (uint32_t*)(b + L.sd);
+  w->scur = (uint32_t*)(b + L.scur);
+  w->touched = (uint32_t*)(b + L.touched);
+  w->sbits = (uint32_t*)(b + L.sbits);
+  w->hist = (uint32_t*)(b + L.hist);
+  w->ring = (uint32_t*)(b + L.ring);
+  w->tasks = (Task*)(b + L.tasks);
+  w->step_ub = (int64_t*)(b + L.step_ub);
+  w->step_off = (uint32_t*)(b + L.step_off);
+  w->ctl = (Ctl*)(b + L.ctl);
+  w->trace = (eic_step*)(b + trace);
+  w->timeline = (unsigned long long*)(b + timeline);
+  static_assert(sizeof(Ctl) <= PinnedSlots::kBytes, "a control block fits a slot");
+  w->ctl_host = (Ctl*)g_mirrors.get();
+  if (!w->ctl_host && cudaMallocHost((void**)&w->ctl_host, sizeof(Ctl)) != cudaSuccess) {
     (void)cudaGetLastError();
     eic_ws_free(w);
     return EIC_ENOMEM;
