@@ -152,7 +152,8 @@ struct Stage {
     };
     uint4 fq[kFuseGroups][kFuseQueue];  // {vertex, distance, row begin, degree}
   };
-  uint32_t fcnt[kFuseGroups][4];  // entries pushed to the local queue, by wave mod 3
+  uint32_t fcnt[kFuseGroups][3];   // entries pushed to the local queue, by wave mod 3
+  uint32_t fstop[kFuseGroups][3];  // set: the group hands on its queue after the wave, by wave mod 3
   uint32_t wf[kMaxWarps][kWarpStage];
 };
 
@@ -1036,7 +1037,9 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
   auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(gn * 32) : "memory"); };
   WarpScr& W = S.w[warp];
   uint4* fq = T.fq[grp];  // the local queue: a ring of kFuseQueue entries
-  uint32_t* fcnt = T.fcnt[grp];
+  // Written in a wave, read by all between its barrier and the next one, and
+  // cleared after that: a warp that is ahead writes the next wave's.
+  uint32_t *fcnt = T.fcnt[grp], *fstop = T.fstop[grp];
   WarpList Fw = {T.wf[warp], 0u, R.first_cnt, R.first_list};
   // the group's share of the items: one block's groups are a grid stride
   // apart, so that few items still reach every SM
@@ -1044,7 +1047,7 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
   uint32_t i0 = min(nitems, (grp * A.nb + qblock(A)) * per);
   const uint32_t i1 = min(nitems, i0 + per);
   const uint32_t np = round1 ? L.push_end - L.push_beg : 0;
-  if (gw == 0 && lane < 4) fcnt[lane] = 0;
+  if (gw == 0 && lane < 3) fcnt[lane] = fstop[lane] = 0;
   group_sync();
   uint32_t spent = 0;
   uint32_t lh = 0, lt = 0, wave = 0;  // the ring's head and tail, the wave mod 3 (the same in every thread of the group)
@@ -1150,7 +1153,7 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
     uint32_t live = 0;  // lanes whose vertex still has the distance it was queued with
     if (!kRoad) {
       spent += (total + 31) / 32;
-      if (spent > kFuseIters && lane == 0) fcnt[3] = 1;
+      if (spent > kFuseIters && lane == 0) fstop[wave] = 1;
     }
     for (uint32_t g0 = 0; g0 < total; g0 += 32) {
       const uint32_t g = g0 + lane;
@@ -1208,9 +1211,11 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
     }
     group_sync();  // the wave's pushes are complete
     lt += min(fcnt[wave], room);
-    if (gw == 0 && lane == 0) fcnt[wave == 0 ? 2 : wave - 1] = 0;  // read by all before this barrier, next used two waves on
+    const bool stop = !kRoad && fstop[wave] && i0 >= i1;
+    const uint32_t last = wave == 0 ? 2 : wave - 1;  // read by all before this barrier, next used two waves on
+    if (gw == 0 && lane == 0) fcnt[last] = fstop[last] = 0;
     wave = wave == 2 ? 0 : wave + 1;
-    if (!kRoad && fcnt[3] && i0 >= i1) {  // long enough alone: the rest goes to the next round
+    if (stop) {  // long enough alone: the rest goes to the next round
       for (uint32_t i = lh + gw * 32; i < lt; i += gn * 32) {
         const bool in = i + lane < lt;
         const uint32_t v = in ? fq[(i + lane) & (kFuseQueue - 1)].x : 0u;
