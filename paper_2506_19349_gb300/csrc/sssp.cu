@@ -406,6 +406,31 @@ __device__ __forceinline__ void emit_tasks(const KArgs& A, const RoundCtx& R, St
   }
 }
 
+// The same by a whole warp, for windows of more than kLaneTasks tasks: a lane
+// that writes the 10,000 tasks of a hub's window alone keeps its warp, and the
+// round, waiting (RMAT 2^25 2.97 -> 2.86 ms, 15 M log-normal 2.00 -> 1.91 ms).
+constexpr uint32_t kLaneTasks = 4;
+__device__ __forceinline__ void emit_tasks_warp(const KArgs& A, const RoundCtx& R, Stage& T, uint32_t b, uint32_t len,
+                                                uint32_t u, uint32_t d) {
+  const uint32_t nt = (len + kTaskLen - 1) / kTaskLen;
+  uint32_t pos = 0, gpos = 0;
+  if (lane_id() == 0) {
+    pos = atomicAdd(&T.tn, nt);
+    const uint32_t in = pos < kStageT ? min(nt, kStageT - pos) : 0;
+    if (nt > in) gpos = atomicAdd(R.tcnt, nt - in) - in;
+  }
+  pos = __shfl_sync(EIC_FULL_MASK, pos, 0);
+  gpos = __shfl_sync(EIC_FULL_MASK, gpos, 0);
+  const uint32_t in_stage = pos < kStageT ? min(nt, kStageT - pos) : 0;
+  for (uint32_t k = lane_id(); k < nt; k += 32) {
+    const Task t = {b + k * kTaskLen, min(kTaskLen, len - k * kTaskLen), u, d};
+    if (k < in_stage)
+      T.tbuf[pos + k] = t;
+    else
+      A.tasks[gpos + k] = t;
+  }
+}
+
 // Successful relaxation of v to nd (old = previous distance): SAP into the
 // next frontier, first insertion into the settled (or first-step) list, and
 // in the first step the running min over high-degree vertices that becomes
@@ -573,8 +598,20 @@ __device__ void round_phase(const KArgs& A, const RoundCtx& R, const Local& L, R
         }
       }
     }
-    if (len > A.heavy_min) {
+    if (len > A.heavy_min && len <= kLaneTasks * kTaskLen) {
       emit_tasks(A, R, T, b, len, u, mode == kModePull ? kNone : val);
+      C.heavy += (len + kTaskLen - 1) / kTaskLen;
+      len = 0;
+    }
+    uint32_t big = __ballot_sync(EIC_FULL_MASK, len > A.heavy_min);
+    while (big) {  // a long window's tasks are written by the whole warp
+      const int src = __ffs(big) - 1;
+      big &= big - 1;
+      emit_tasks_warp(A, R, T, __shfl_sync(EIC_FULL_MASK, b, src), __shfl_sync(EIC_FULL_MASK, len, src),
+                      __shfl_sync(EIC_FULL_MASK, u, src),
+                      __shfl_sync(EIC_FULL_MASK, mode == kModePull ? kNone : val, src));
+    }
+    if (len > A.heavy_min) {
       C.heavy += (len + kTaskLen - 1) / kTaskLen;
       len = 0;
     }
