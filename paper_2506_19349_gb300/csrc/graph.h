@@ -26,6 +26,10 @@ struct Ctl {
   uint32_t s_int;  // internal id of the source (0xFFFFFFFF: isolated source)
   uint32_t push_beg, push_end;  // settled-list range pushed in the step's first round
   uint32_t pull_on, pull_cnt, extra_s;
+  uint32_t f2;  // the boundary waits for f2_bins over settled-list entries [f2_beg, f2_end)
+  uint32_t f2_beg, f2_end;
+  int64_t f2_wl, f2_st0;
+  uint64_t f2_span;
   uint32_t pull_sweep;  // the pull set is swept in vertex order (pull_cnt = all vertices; the round takes the unsettled ones)
   uint32_t step_off_cur;  // settled-list offset where the current step's vertices start
   // private to the step-boundary block

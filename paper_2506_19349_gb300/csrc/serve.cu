@@ -121,6 +121,7 @@ struct eic_server {
   eic_params p{};
   uint32_t groups = 0, nb = 0, block = 0, cap = 0;  // groups (slots) at most, blocks per group at that count
   uint32_t gmax = 0;                                 // co-resident blocks of the serving kernel
+  bool wide = false;                                 // a resident graph has weights of 2^20 and above
   uint32_t launch_groups = 0;                        // groups of the running (or last) launch
   uint64_t idle_ns = 0;
   SlotPool pool;
@@ -176,6 +177,7 @@ struct eic_server {
     const uint32_t sl = p.max_spin_log2 > kServeSpinLog2 ? p.max_spin_log2 : kServeSpinLog2;
     a.max_spin = 1ull << sl;
     a.groups = g;
+    a.wide = wide;
     a.idle_ns = idle_ns;
     a.poll_ns = kPollUs * 1000ull;
     a.widen_at = g < groups ? 2ull * g : 0ull;
@@ -360,6 +362,7 @@ int eic_server_create(const eic_graph* const* graphs, uint32_t num_graphs, const
     q.G = G;
     uint32_t shift = 0;
     const uint32_t bits = ring_layout(G.maxw, &shift);
+    s->wide |= shift != 0;
     q.ring_mask = (1u << bits) - 1u;
     q.ring_shift = shift;
     q.task_cap = (uint32_t)(G.two_m / kHeavyMinFloor + 2);
@@ -374,7 +377,7 @@ int eic_server_create(const eic_graph* const* graphs, uint32_t num_graphs, const
     max_n = std::max<uint64_t>(max_n, G.n);
   }
   uint32_t gmax = 0;
-  if ((rc = eic_serve_grid((int)s->block, &gmax))) goto fail;
+  if ((rc = eic_serve_grid((int)s->block, s->wide, &gmax))) goto fail;
   {
     uint32_t groups = cfg.groups ? cfg.groups : std::max(1u, gmax / 8);
     groups = std::min(groups, gmax);

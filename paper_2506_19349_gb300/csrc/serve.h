@@ -45,6 +45,7 @@ struct ServeArgs {
   const BatchSlot* slot;          // [groups]
   uint32_t num_graphs, cap, nb;   // graphs; ring entries; blocks per group
   uint32_t groups;
+  uint32_t wide;                  // a resident graph has weights of 2^20 and above
   uint32_t alpha;
   double beta;
   uint32_t st_num, gap_shift, heavy_min, flags, step_cap;
@@ -61,8 +62,8 @@ struct ServeArgs {
 // threads, cooperatively, on stream. Returns an EIC_* status.
 int eic_serve_launch(const ServeArgs& args, uint32_t groups, uint32_t block, cudaStream_t stream);
 
-// Co-resident blocks of the serving kernel at this block size.
-int eic_serve_grid(int block, uint32_t* grid);
+// Co-resident blocks of the serving kernel at this block size (wide: for graphs with weights of 2^20 and above).
+int eic_serve_grid(int block, bool wide, uint32_t* grid);
 
 // The step-width scaling (gap_shift, from `from` upwards while it helps by 2%,
 // up to 8) that runs (g, source) fastest in a group of nb blocks: `copies`

@@ -225,6 +225,10 @@ struct BState {
   int64_t hub[kStepHist];    // ub of step j at j % kStepHist
   uint32_t hoff[kStepHist];  // step j's first settled-list entry
   uint32_t j0;
+  // a boundary that waits for f2_bins
+  uint64_t p_sumd;
+  int64_t p_gap, p_st0, p_st1;
+  uint32_t p_highd, p_settled;
 };
 
 struct Counters {  // one thread's counts over the query (added to the 64-bit totals at its end)
@@ -945,34 +949,26 @@ __device__ __forceinline__ int64_t st_candidate(uint32_t k, uint64_t span, uint3
 }
 
 
-// Function 2 for weights of 2^20 and above (one block), with D(x') summed
-// exactly from the settled list: over the entries of the steps
-// j (from j0 to step) that end above wl, the vertex at distance d >= wl adds
-// its degree to bin 1 + k_d, k_d the last candidate k with x_k <= d (-1 if
-// none); after a suffix sum, D(x_k) is bin 1 + k for x_k >= wl and bin 0 for a
-// candidate clamped to wl. The bins are in shared memory, or in the ring
-// (2^20 slots, unused for such weights) when ST_NUM is large.
-__device__ __forceinline__ int64_t block_st_exact(const KArgs& A, S3Scr& S, int64_t ub, uint64_t sumd_ub,
-                                                  int64_t gap_lb, int64_t gap_ub_raw, int64_t y, int64_t st0,
-                                                  int64_t st1, uint32_t j0, uint32_t step, uint32_t send) {
-  __shared__ uint32_t s_beg;
-  const uint32_t t = threadIdx.x, nt = blockDim.x;
-  const int64_t maxw = A.G.maxw;
-  if (sumd_ub >= A.G.m || gap_lb == maxw) return ub;
-  if (gap_ub_raw == maxw) return ub - maxw;
-  const int64_t wl = ub - maxw > 0 ? ub - maxw : 0;
-  const uint64_t nbins = (uint64_t)A.st_num + 2;
-  const bool sh = nbins <= kSufMax;
-  uint32_t* bins = sh ? S.suf : A.ring;  // (a degree sum is at most 2m < 2^32)
-  for (uint64_t q = t; q < nbins; q += nt) bins[q] = 0u;
-  if (t == 0) {
-    uint32_t j = j0;
-    while (j <= step && __ldcg(&A.step_ub[j]) <= wl) ++j;
-    s_beg = j <= step ? __ldcg(&A.step_off[j]) : send;
-  }
+// Function 2 for weights of 2^20 and above, with D(x') summed exactly from the
+// settled list: over the entries of the steps that end above wl, the vertex at
+// distance d >= wl adds its degree to bin 1 + k_d, k_d the last candidate k
+// with x_k <= d (-1 if none); after a suffix sum, D(x_k) is bin 1 + k for x_k >=
+// wl and bin 0 for a candidate clamped to wl. All blocks of the query fill the
+// bins (the ring's words, unused for such weights) between two grid barriers:
+// one block alone took 95, 185 and 271 us in three steps of an RMAT graph of
+// 250 k vertices. A block counts in shared memory first when it has at least
+// as many entries as there are bins.
+__device__ __forceinline__ void f2_bins(const KArgs& A, S3Scr& S, const Ctl* c) {
+  const uint32_t t = threadIdx.x, nt = blockDim.x, n0 = qblock(A) * nt, stride = A.nb * nt;
+  const uint32_t beg = __ldcg(&c->f2_beg), end = __ldcg(&c->f2_end);
+  const int64_t wl = __ldcg(&c->f2_wl), st0 = __ldcg(&c->f2_st0);
+  const uint64_t span = __ldcg(&c->f2_span);
+  const uint32_t nbins = A.st_num + 2;
+  const bool sh = nbins <= kSufMax && (end - beg) / A.nb >= nbins;
+  if (sh)
+    for (uint32_t q = t; q < nbins; q += nt) S.suf[q] = 0u;
   __syncthreads();
-  const uint64_t span = (uint64_t)(st1 - st0);
-  for (uint32_t i = s_beg + t; i < send; i += nt) {
+  for (uint32_t i = beg + n0 + t; i < end; i += stride) {
     const int64_t d = ld_list(&A.sd[i]);
     if (d < wl) continue;
     const uint32_t dg = __ldg(&A.G.dvals[degree_rank(A.G, ld_list(&A.sid[i]))]);
@@ -982,15 +978,33 @@ __device__ __forceinline__ int64_t block_st_exact(const KArgs& A, S3Scr& S, int6
     else if (span == 0)
       cnt = nbins - 1;
     else
-      cnt = min(((uint64_t)(d - st0 + 1) * A.st_num + span - 1) / span, nbins - 1);
-    atomicAdd(&bins[cnt], dg);
+      cnt = min(((uint64_t)(d - st0 + 1) * A.st_num + span - 1) / span, (uint64_t)nbins - 1);
+    atomicAdd(sh ? &S.suf[cnt] : &A.ring[cnt], dg);  // (a degree sum is at most 2m < 2^32)
   }
   __syncthreads();
+  if (sh) {
+    for (uint32_t q = t; q < nbins; q += nt)
+      if (S.suf[q]) atomicAdd(&A.ring[q], S.suf[q]);
+    __syncthreads();
+  }
+}
+
+// The same out of line for the batch and serving kernels, which hold their
+// arguments in shared memory: inlined there it costs their query loop registers.
+__device__ __noinline__ void f2_bins_call(const KArgs& A, S3Scr& S, const Ctl* c) { f2_bins(A, S, c); }
+
+// The candidate of the bins for an ST_NUM above the shared-memory window (one
+// block): suffix sums in place, every profit in double precision.
+__device__ __noinline__ int64_t block_st_bins(uint32_t* bins, uint32_t st_num, uint32_t maxw, uint64_t two_m, S3Scr& S,
+                                              int64_t ub, uint64_t sumd_ub, int64_t y, int64_t st0, int64_t st1) {
+  const uint32_t t = threadIdx.x, nt = blockDim.x;
+  const int64_t wl = ub - (int64_t)maxw > 0 ? ub - (int64_t)maxw : 0;
+  const uint64_t nbins = (uint64_t)st_num + 2, span = (uint64_t)(st1 - st0);
   // suffix sums: chunk totals, a scan over the chunks, then within the chunks
   const uint64_t cs = (nbins + nt - 1) / nt;
-  const uint64_t q0 = t * cs, q1 = min(nbins, q0 + cs);
+  const uint64_t q0 = min(nbins, t * cs), q1 = min(nbins, q0 + cs);
   uint32_t mine = 0;
-  for (uint64_t q = q0; q < q1; ++q) mine += sh ? bins[q] : __ldcg(&bins[q]);
+  for (uint64_t q = q0; q < q1; ++q) mine += __ldcg(&bins[q]);
   S.part[t] = mine;
   __syncthreads();
   for (uint32_t o = 1; o < nt; o <<= 1) {
@@ -1001,39 +1015,25 @@ __device__ __forceinline__ int64_t block_st_exact(const KArgs& A, S3Scr& S, int6
   }
   uint32_t acc = t + 1 < nt ? S.part[t + 1] : 0;
   for (uint64_t q = q1; q > q0; --q) {
-    acc += sh ? bins[q - 1] : __ldcg(&bins[q - 1]);
-    if (sh)
-      bins[q - 1] = acc;
-    else
-      __stcg(&bins[q - 1], acc);
+    acc += __ldcg(&bins[q - 1]);
+    __stcg(&bins[q - 1], acc);
   }
   __syncthreads();
   double best = 0.0;
   uint32_t bk = 0xFFFFFFFFu;
-  const uint32_t gsh = (A.st_num & (A.st_num - 1)) == 0 ? __ffs(A.st_num) - 1 : 32u;
-  for (uint32_t k = t; k <= A.st_num; k += nt) {
-    const int64_t x = st_candidate(k, span, A.st_num, gsh, st0);
+  const uint32_t gsh = (st_num & (st_num - 1)) == 0 ? __ffs(st_num) - 1 : 32u;
+  for (uint32_t k = t; k <= st_num; k += nt) {
+    const int64_t x = st_candidate(k, span, st_num, gsh, st0);
     if (x >= ub) continue;
-    const uint64_t q = x >= wl ? (uint64_t)k + 1 : 0;
-    const uint32_t dsum = sh ? bins[q] : __ldcg(&bins[q]);
-    const double p = dev_profit(x, ub, y, dsum, sumd_ub, A.G.maxw, A.G.two_m);
+    const uint32_t dsum = __ldcg(&bins[x >= wl ? (uint64_t)k + 1 : 0]);
+    const double p = dev_profit(x, ub, y, dsum, sumd_ub, maxw, two_m);
     if (p > best) {
       best = p;
       bk = k;
     }
   }
   const uint32_t k = block_argmax(S, best, bk);
-  if (k == 0xFFFFFFFFu) return ub;
-  return st_candidate(k, span, A.st_num, gsh, st0);
-}
-
-// The same out of line, for the batch and serving kernels: inlined there it
-// costs their query loop registers (and their speed), while the single-query
-// kernel is not affected either way.
-__device__ __noinline__ int64_t block_st_exact_call(const KArgs& A, S3Scr& S, int64_t ub, uint64_t sumd_ub,
-                                                    int64_t gap_lb, int64_t gap_ub_raw, int64_t y, int64_t st0,
-                                                    int64_t st1, uint32_t j0, uint32_t step, uint32_t send) {
-  return block_st_exact(A, S, ub, sumd_ub, gap_lb, gap_ub_raw, y, st0, st1, j0, step, send);
+  return k == 0xFFFFFFFFu ? ub : st_candidate(k, span, st_num, gsh, st0);
 }
 
 // A fused round: the FUSED local iterations of Section 4.1 (bucket fusion), in
@@ -1311,7 +1311,7 @@ __device__ __forceinline__ void f2_load(const KArgs& A, S3Scr& S, const F2Window
 // candidate with the largest positive profit, or ub. D(x') = sumD(x') -
 // sumD(ub), the degree sum of the settled vertices with x' <= dist < ub, x' =
 // max(x, ub - maxW), is a suffix sum of the ring (one slot per distance: maxW <
-// 2^20; wider weights go through block_st_exact).
+// 2^20), or, for wider weights, of f2_bins' bins (w.cs = 0: one chunk per bin).
 //
 // The profit is specified in double precision, of which this GPU has two
 // operations per clock and SM: ST_NUM candidates with three divisions each cost
@@ -1319,7 +1319,7 @@ __device__ __forceinline__ void f2_load(const KArgs& A, S3Scr& S, const F2Window
 // pulled, an exact integer comparison (each double operation rounds
 // monotonically, so pushed <= pulled there means profit <= 0 here), and, of
 // these, those whose single-precision estimate comes within twice its error
-// bound of the best. The estimate's error is at most 20 roundings of
+// bound of the best. The estimate's error is at most 26 roundings of
 // 2^-24 of pushed <= pushed(x = wl), which bounds every term; e takes 32.
 // Function 2 went from 5.6 to 2.5 us a step on a uniform graph of 2^14 vertices.
 __device__ int64_t block_compute_st(const KArgs& A, S3Scr& S, const F2Window& w, int64_t ub, uint64_t sumd_ub,
@@ -1366,7 +1366,9 @@ __device__ int64_t block_compute_st(const KArgs& A, S3Scr& S, const F2Window& w,
       if ((xp > lo ? xp : lo) == xc) return false;
     }
     const uint32_t i = (uint32_t)(xc - w.wl);
-    if (w.cs <= 1) {
+    if (w.cs == 0) {
+      dsum = S.suf[x >= w.wl ? k + 1 : 0];
+    } else if (w.cs == 1) {
       dsum = S.suf[i];
     } else {
       const uint32_t c = i / w.cs, ce = min(w.slots, (c + 1) * w.cs);
@@ -1440,8 +1442,13 @@ __device__ int64_t block_compute_st(const KArgs& A, S3Scr& S, const F2Window& w,
 // barriers, and double precision is used only where a single-precision
 // estimate cannot decide. A boundary went from 10.8 to 7.2 us on the 4096^2
 // grid, from 10.9 to 5.8 us on a uniform graph of 2^14 vertices.
-template <bool kExactInline>
-__device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Local& L, uint32_t rounds_in_step) {
+//
+// With weights of 2^20 and above and Function 2 to be evaluated, it stops
+// before that and asks all blocks for f2_bins (c->f2); it then runs again with
+// `second` set and goes on from there.
+template <bool kWide>
+__device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Local& L, uint32_t rounds_in_step,
+                              bool second) {
   Ctl* c = A.ctl;
   __shared__ HighdScr s_h;
   __shared__ uint32_t s_rw[32];
@@ -1453,8 +1460,45 @@ __device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Loca
   const uint32_t t = threadIdx.x, nt = blockDim.x, lane = lane_id(), warp = t >> 5;
   const int64_t lb = L.lb, ub = L.ub, maxw = G.maxw;
   const uint32_t k = L.step;
-  uint32_t settled_now = 0, maxd1 = 0;
+  uint32_t settled_now = 0, maxd1 = 0, highd_ub;
   unsigned long long acc = 0;
+  uint64_t sumd_ub;
+  int64_t gap_raw, st0, st1, nst = ub;
+  // this thread's run of the window's chunk sums, summed from the end of the warp
+  auto window_sums = [&](const F2Window& w) -> uint32_t {
+    const uint32_t per = (w.chunks + nt - 1) / nt, b = min(w.chunks, t * per), e = min(w.chunks, b + per);
+    uint32_t x = 0;
+    for (uint32_t q = b; q < e; ++q) x += S.suf[q];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t z = __shfl_down_sync(EIC_FULL_MASK, x, o);
+      if (lane + o < 32) x += z;
+    }
+    if (lane == 0) s_rw[warp] = x;
+    return x;
+  };
+  if (kWide && second) {
+    sumd_ub = B.p_sumd;
+    highd_ub = B.p_highd;
+    gap_raw = B.p_gap;
+    st0 = B.p_st0;
+    st1 = B.p_st1;
+    F2Window w;
+    w.wl = ub > maxw ? ub - maxw : 0;
+    w.slots = 0;
+    w.cs = 0;
+    w.chunks = A.st_num + 2;
+    const int64_t y = ub + (gap_raw << A.gap_shift);
+    if (w.chunks <= kSufMax) {
+      for (uint32_t q = t; q < w.chunks; q += nt) S.suf[q] = __ldcg(&A.ring[q]);
+      __syncthreads();
+      const uint32_t wsuf = window_sums(w);
+      __syncthreads();
+      nst = block_compute_st(A, S, w, ub, sumd_ub, y, st0, st1, wsuf, s_rw);
+    } else {
+      nst = block_st_bins(A.ring, A.st_num, G.maxw, G.two_m, S, ub, sumd_ub, y, st0, st1);
+    }
+  } else {
   if (t == 0) {
     settled_now = __ldcg(&c->settled_cnt);
     acc = __ldcg(&c->acc_deg);
@@ -1504,7 +1548,7 @@ __device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Loca
     }
   }
   __syncthreads();
-  const uint64_t sumd_ub = s_sumd;
+  sumd_ub = s_sumd;
   if (s_done) {
     if (t == 0) {
       c->done = 1;
@@ -1512,56 +1556,62 @@ __device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Loca
     }
     return;
   }
-  // this thread's run of the window's chunk sums, summed from the end of the warp
-  auto window_sums = [&]() -> uint32_t {
-    const uint32_t per = (w.chunks + nt - 1) / nt, b = min(w.chunks, t * per), e = min(w.chunks, b + per);
-    uint32_t x = 0;
-    for (uint32_t q = b; q < e; ++q) x += S.suf[q];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t z = __shfl_down_sync(EIC_FULL_MASK, x, o);
-      if (lane + o < 32) x += z;
-    }
-    if (lane == 0) s_rw[warp] = x;
-    return x;
-  };
   highd_cross(A.hist, G.dvals, G.D, hp, s_h);
-  uint32_t wsuf = early ? window_sums() : 0u;
+  uint32_t wsuf = early ? window_sums(w) : 0u;
   __syncthreads();
-  const uint32_t highd_ub = s_h.highd;
-  int64_t gap_raw = dev_gap_quick(sumd_ub, highd_ub, G.two_m, A.alpha, A.beta, G.rtow);
+  highd_ub = s_h.highd;
+  gap_raw = dev_gap_quick(sumd_ub, highd_ub, G.two_m, A.alpha, A.beta, G.rtow);
   if (gap_raw < 0) {  // (the same in every thread)
     if (t == 0) s_gap = dev_gap(sumd_ub, highd_ub, G.two_m, A.alpha, A.beta, G.rtow);
     __syncthreads();
     gap_raw = s_gap;
   }
-  const int64_t st0 = k == 1 ? ub : B.st0, st1 = B.st1 < 0 && sumd_ub <= G.m ? ub : B.st1;
-  const int64_t nlb = ub, nub = ub + (gap_raw << A.gap_shift);
-  int64_t nst = nlb;
+  st0 = k == 1 ? ub : B.st0;
+  st1 = B.st1 < 0 && sumd_ub <= G.m ? ub : B.st1;
   if (!(A.flags & EIC_FLAG_NO_PULL) && sumd_ub < G.m && gap_lb != maxw) {
     if (gap_raw == maxw) {
       nst = ub - maxw;
-    } else if (A.ring_shift == 0) {
+    } else if (!kWide || A.ring_shift == 0) {
       if (!early) {
         f2_load(A, S, w);
         __syncthreads();
-        wsuf = window_sums();
+        wsuf = window_sums(w);
         __syncthreads();
       }
-      nst = block_compute_st(A, S, w, ub, sumd_ub, nub, st0, st1, wsuf, s_rw);
-    } else {
-      nst = kExactInline
-                ? block_st_exact(A, S, ub, sumd_ub, gap_lb, gap_raw, nub, st0, st1, B.j0, k, s_settled)
-                : block_st_exact_call(A, S, ub, sumd_ub, gap_lb, gap_raw, nub, st0, st1, B.j0, k, s_settled);
+      nst = block_compute_st(A, S, w, ub, sumd_ub, ub + (gap_raw << A.gap_shift), st0, st1, wsuf, s_rw);
+    } else {  // ask for the bins: the settled steps j that end above wl
+      for (uint32_t q = t; q < A.st_num + 2; q += nt) __stcg(&A.ring[q], 0u);
+      __syncthreads();  // every thread is done with the controller's state
+      if (t == 0) {
+        B.p_sumd = sumd_ub;
+        B.p_highd = highd_ub;
+        B.p_gap = gap_raw;
+        B.p_st0 = st0;
+        B.p_st1 = st1;
+        B.p_settled = s_settled;
+        const int64_t wl = ub > maxw ? ub - maxw : 0;
+        uint32_t j = B.j0;
+        while (j <= k && __ldcg(&A.step_ub[j]) <= wl) ++j;
+        c->f2_beg = j <= k ? __ldcg(&A.step_off[j]) : s_settled;
+        c->f2_end = s_settled;
+        c->f2_wl = wl;
+        c->f2_st0 = st0;
+        c->f2_span = (uint64_t)(st1 - st0);
+        c->s2_done = 0;
+        c->f2 = 1;
+      }
+      return;
     }
   }
+  }
+  const int64_t nlb = ub, nub = ub + (gap_raw << A.gap_shift);
   if (t >= 32) {
     if (A.ring_shift == 0) {  // zero the ring slots the next statistics pass fills: [max(nlb, nub - maxW), nub)
       const int64_t zl = nub - maxw > nlb ? nub - maxw : nlb;
       for (int64_t q = zl + (t - 32); q < nub; q += nt - 32) __stcg(&A.ring[(uint32_t)q & A.ring_mask], 0u);
     }
   } else if (t == 0) {
-    settled_now = s_settled;
+    settled_now = kWide && second ? B.p_settled : s_settled;
     A.step_off[k + 1] = settled_now;
     B.hoff[(k + 1) % kStepHist] = settled_now;
     uint32_t scnt = settled_now;
@@ -1644,6 +1694,7 @@ __device__ void step_boundary(const KArgs& A, PhaseScr& P, BState& B, const Loca
     c->acc_deg = 0;
     c->acc_maxd1 = 0;
     c->s2_done = 0;
+    c->f2 = 0;
     c->done = 0;  // the control values are published by the grid barrier's release
   }
   __syncthreads();  // every thread is done with the controller's state of this step
@@ -1715,7 +1766,9 @@ struct QueryShared {
 // The query loop of Algorithm 1 run by the A.nb blocks of one query: rounds
 // of a step (item phase, task phase), statistics pass, step boundary, until
 // termination. ticket is the block's arrival ticket of the query's barrier.
-template <uint32_t kPullFast, uint32_t kRelaxIlp>
+// kWide: the query's graph may have weights of 2^20 and above. Without that
+// code the other graphs' queries are 2 to 4% faster (registers).
+template <uint32_t kPullFast, uint32_t kRelaxIlp, bool kWide>
 __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ticket) {
   PhaseScr& P = Q.P;
   Stage& T = Q.T;
@@ -1956,8 +2009,12 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ti
         }
         __syncthreads();
       }
-      if (threadIdx.x == 0) red_release_add_u32(&c->s2_done, 1u);  // releases the block's statistics
-      if (qb == 0) {  // block 0 waits (bounded) for every block's statistics
+    }
+    // The boundary, by block 0 once every block has released its part. With wide weights it may first ask all
+    // blocks for Function 2's bins.
+    for (bool second = false;; second = true) {
+      if (threadIdx.x == 0) red_release_add_u32(&c->s2_done, 1u);
+      if (qb == 0) {  // block 0 waits (bounded) for every block's part
         if (threadIdx.x == 0) {
           uint64_t spins = 0;
           sh_last = 1;
@@ -1971,11 +2028,20 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ti
           tl_mark(A, 4, L.rid);
         }
         __syncthreads();
-        if (sh_last) step_boundary<(kRelaxIlp >= 2)>(A, P, B, L, rin);  // (the single-query shape inlines)
+        if (sh_last) step_boundary<kWide>(A, P, B, L, rin, second);
         if (threadIdx.x == 0) tl_mark(A, 5, L.rid);
       }
+      alive = grid_barrier(&c->bar, &ticket, A.nb, A.max_spin, &c->status);
+      if (!kWide || !alive || A.ring_shift == 0) break;
+      if (threadIdx.x == 0) sh_last = __ldcg(&c->f2);
+      __syncthreads();
+      if (!sh_last) break;
+      if constexpr (kRelaxIlp >= 2)
+        f2_bins(A, P.s3, c);
+      else
+        f2_bins_call(A, P.s3, c);
     }
-    if (!grid_barrier(&c->bar, &ticket, A.nb, A.max_spin, &c->status)) break;
+    if (!alive) break;
     if (qb == 0 && threadIdx.x == 0) tl_mark(A, 3, L.rid);
     read_ctl(c, L);
     if (L.done) break;
@@ -1995,10 +2061,11 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ti
   if (qb == 0 && threadIdx.x == 0 && A.status_out) *A.status_out = ld_volatile_int(&c->status);
 }
 
+template <bool kWide>
 __global__ void __launch_bounds__(kMaxBlock, 2) k_eic(KArgs A) {
   __shared__ QueryShared Q;
   unsigned long long ticket = 0;  // (k_init zeroed the arrival count)
-  run_query<kPullFastSingle, kRelaxIlpSingle>(A, Q, ticket);
+  run_query<kPullFastSingle, kRelaxIlpSingle, kWide>(A, Q, ticket);
 }
 
 // Control block of a new query (one thread): the source's distance, the
@@ -2022,6 +2089,7 @@ __device__ void ctl_init(const KArgs& A) {
   c->st = 0;
   c->lb0 = 0;
   c->step = 1;
+  c->f2 = 0;
   c->done = si == EIC_INF ? 1u : 0u;
   c->push_beg = c->push_end = 0;
   c->pull_on = c->pull_cnt = c->extra_s = 0;
@@ -2153,6 +2221,7 @@ __device__ void query_output(const KArgs& A) {
 // with its own scratch and a barrier over its nb blocks, writes the output,
 // and claims again. A group stops at its first query with a non-OK status
 // (its barrier state is then unreliable); the other groups carry on.
+template <bool kWide>
 __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_batch(BatchArgs P) {
   __shared__ QueryShared Q;
   __shared__ KArgs sA;
@@ -2212,7 +2281,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_batch(BatchArgs P) {
     }
     __syncthreads();
     if (!query_setup(sA, ticket)) break;
-    run_query<kPullFastGroup, kRelaxIlpGroup>(sA, Q, ticket);
+    run_query<kPullFastGroup, kRelaxIlpGroup, kWide>(sA, Q, ticket);
     __syncthreads();
     if (ld_volatile_int(&c->status) != 0) break;
     query_output(sA);
@@ -2282,6 +2351,7 @@ constexpr unsigned long long kRetry = ~0ull - 1;      // nothing yet: the group 
 // requests wait unclaimed (each after its current request; the host then
 // relaunches with more groups). A group stops at its first failing request
 // (whose completion carries the error) and counts as idle from then on.
+template <bool kWide>
 __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_serve(ServeArgs P) {
   __shared__ QueryShared Q;
   __shared__ KArgs sA;
@@ -2397,7 +2467,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_serve(ServeArgs P) {
     }
     __syncthreads();
     if (!query_setup(sA, ticket)) break;
-    run_query<kPullFastGroup, kRelaxIlpGroup>(sA, Q, ticket);
+    run_query<kPullFastGroup, kRelaxIlpGroup, kWide>(sA, Q, ticket);
     __syncthreads();
     if (ld_volatile_int(&c->status) != 0) break;
     query_output(sA);
@@ -2492,7 +2562,8 @@ int launch_shape(Workspace* ws, int block) {
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
   if (!coop) return EIC_ECUDA;
-  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eic, block, 0));
+  const bool wide = ws->ring_shift != 0;
+  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wide ? k_eic<true> : k_eic<false>, block, 0));
   if (per_sm < 1) return EIC_ECUDA;
   ws->grid = sms * per_sm;
   ws->block = block;
@@ -2563,7 +2634,8 @@ int enqueue_query(eic_graph* g, uint32_t s, uint32_t* dist, uint32_t* parent, co
   EIC_CUDA_TRY(cudaGetLastError());
   void* args[] = {&A};
   if (ev0) EIC_CUDA_TRY(cudaEventRecord(ev0, st));
-  EIC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_eic, dim3(grid), dim3(block), args, 0, st));
+  EIC_CUDA_TRY(cudaLaunchCooperativeKernel(w.ring_shift ? (const void*)k_eic<true> : (const void*)k_eic<false>, dim3(grid),
+                                           dim3(block), args, 0, st));
   if (ev1) EIC_CUDA_TRY(cudaEventRecord(ev1, st));
   k_output<<<4 * grid, 256, 0, st>>>(g->dg, w.idist, s, dist);
   EIC_CUDA_TRY(cudaGetLastError());
@@ -2770,13 +2842,14 @@ int eic_sssp(const eic_graph* gc, uint32_t source, uint32_t* dist, uint32_t* par
 
 namespace {
 
-int batch_grid(int block, uint32_t* grid) {
+int batch_grid(int block, bool wide, uint32_t* grid) {
   int dev = 0, sms = 0, per_sm = 0, coop = 0;
   EIC_CUDA_TRY(cudaGetDevice(&dev));
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
   if (!coop) return EIC_ECUDA;
-  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eic_batch, block, 0));
+  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wide ? k_eic_batch<true> : k_eic_batch<false>,
+                                                             block, 0));
   if (per_sm < 1) return EIC_ECUDA;
   *grid = (uint32_t)(sms * per_sm);
   return EIC_OK;
@@ -2813,6 +2886,7 @@ struct eic_batch {
   int* h_status = nullptr;
   uint32_t* d_queue = nullptr;
   bool use_graph = true;
+  bool wide = false;  // a graph of the batch has weights of 2^20 and above
   cudaGraphExec_t exec = nullptr;
   double tuned_ms = 0.0;
 };
@@ -2838,7 +2912,7 @@ uint32_t groups_that_fit(eic_batch* b, uint32_t want) {
 // most the co-resident grid.
 int batch_configure(eic_batch* b, uint32_t groups, uint32_t block, uint32_t nb_force = 0) {
   uint32_t gmax = 0;
-  int rc = batch_grid((int)block, &gmax);
+  int rc = batch_grid((int)block, b->wide, &gmax);
   if (rc) return rc;
   if (nb_force) {
     if (nb_force > gmax) nb_force = gmax;
@@ -2903,8 +2977,8 @@ int batch_enqueue(eic_batch* b, cudaStream_t st) {
     k_batch_prep<<<(cover + 255) / 256, 256, 0, st>>>(P, b->groups);
     EIC_CUDA_TRY(cudaGetLastError());
     void* args[] = {&P};
-    EIC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_eic_batch, dim3(b->groups * b->nb), dim3(b->block), args,
-                                             0, st));
+    EIC_CUDA_TRY(cudaLaunchCooperativeKernel(b->wide ? (const void*)k_eic_batch<true> : (const void*)k_eic_batch<false>,
+                                             dim3(b->groups * b->nb), dim3(b->block), args, 0, st));
   }
   for (const auto& t : b->trivial) {  // no edges: only the source is reachable
     EIC_CUDA_TRY(cudaMemsetAsync(t.dist, 0xFF, (uint64_t)t.n * 4, st));
@@ -2962,6 +3036,7 @@ int batch_create(const eic_graph* const* graphs, const uint32_t* sources, uint32
     q.s = sources[i];
     uint32_t shift = 0;
     const uint32_t bits = ring_layout(G.maxw, &shift);
+    b->wide |= shift != 0;
     q.ring_mask = (1u << bits) - 1u;
     q.ring_shift = shift;
     q.task_cap = (uint32_t)(G.two_m / kHeavyMinFloor + 2);
@@ -3159,7 +3234,7 @@ int eic_batch_tune(eic_batch* b, void* stream, eic_batch_config* best) {
       return EIC_OK;
     };
     uint32_t gmax = 0;
-    if ((rc = batch_grid((int)b->block, &gmax))) return rc;
+    if ((rc = batch_grid((int)b->block, b->wide, &gmax))) return rc;
     // pass 1: group counts (divisors of the grid and powers of two), from the
     // most groups down, until two in a row are 20% slower than the best
     std::vector<uint32_t> cand;
@@ -3336,7 +3411,7 @@ int na_setup(NaDevice& d, cudaStream_t st) {
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
   if (!coop) return EIC_ECUDA;
-  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eic, kDefaultBlock, 0));
+  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eic<false>, kDefaultBlock, 0));
   if (per_sm < 1) return EIC_ECUDA;
   unsigned char* base = (unsigned char*)ptr;
   EIC_CUDA_TRY(cudaMemsetAsync(base + kNaCtl, 0, sizeof(Ctl), st));
@@ -3417,7 +3492,7 @@ extern "C" int eic_sssp_noalloc(const eic_graph* gc, uint32_t source, uint32_t* 
     k_init<<<64, 256, 0, st>>>(A);
     EIC_CUDA_TRY(cudaGetLastError());
     void* args[] = {&A};
-    EIC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_eic, dim3(nd.grid), dim3(kDefaultBlock), args, 0, st));
+    EIC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_eic<false>, dim3(nd.grid), dim3(kDefaultBlock), args, 0, st));
     k_output<<<4 * nd.grid, 256, 0, st>>>(G, A.dist, source, dist);
     EIC_CUDA_TRY(cudaGetLastError());
     return EIC_OK;
@@ -3434,13 +3509,14 @@ extern "C" int eic_sssp_noalloc(const eic_graph* gc, uint32_t source, uint32_t* 
 
 // ------------------------------------------------------------ serving launch
 
-int eic_serve_grid(int block, uint32_t* grid) {
+int eic_serve_grid(int block, bool wide, uint32_t* grid) {
   int dev = 0, sms = 0, per_sm = 0, coop = 0;
   EIC_CUDA_TRY(cudaGetDevice(&dev));
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   EIC_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
   if (!coop) return EIC_ECUDA;
-  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eic_serve, block, 0));
+  EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wide ? k_eic_serve<true> : k_eic_serve<false>,
+                                                             block, 0));
   if (per_sm < 1) return EIC_ECUDA;
   *grid = (uint32_t)(sms * per_sm);
   return EIC_OK;
@@ -3451,8 +3527,8 @@ int eic_serve_launch(const ServeArgs& args, uint32_t groups, uint32_t block, cud
   EIC_CUDA_TRY(cudaGetLastError());
   ServeArgs a = args;
   void* kargs[] = {&a};
-  EIC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_eic_serve, dim3(groups * args.nb), dim3(block), kargs, 0,
-                                           stream));
+  EIC_CUDA_TRY(cudaLaunchCooperativeKernel(args.wide ? (const void*)k_eic_serve<true> : (const void*)k_eic_serve<false>,
+                                           dim3(groups * args.nb), dim3(block), kargs, 0, stream));
   return EIC_OK;
 }
 
