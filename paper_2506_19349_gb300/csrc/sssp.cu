@@ -359,6 +359,36 @@ __device__ __forceinline__ uint32_t gallop_w(const uint2* __restrict__ adj, uint
   return lower_bound_w(adj, lo + 1, hi, t);
 }
 
+// The same for windows that mostly end within four entries: the weights of the
+// first four are read at once. (RMAT 2^25 2779 -> 2730 us, 15 M log-normal
+// 1885 -> 1863 us; a window's average length there is 1.3 entries.)
+__device__ __forceinline__ uint32_t gallop4_w(const uint2* __restrict__ adj, uint32_t p, uint32_t e, int64_t t) {
+  if (t <= 1 || p >= e) return p;
+  uint32_t w[4], c = 0;
+#pragma unroll
+  for (uint32_t k = 0; k < 4; ++k) w[k] = p + k < e ? ld_stream_w(&adj[p + k]) : 0xFFFFFFFFu;
+#pragma unroll
+  for (uint32_t k = 0; k < 4; ++k) c += p + k < e && (int64_t)w[k] < t ? 1u : 0u;
+  if (c < 4) return p + c;
+  uint32_t lo = p + 3;  // weight at lo < t
+  uint32_t hi;
+  uint64_t step = 1;
+  for (;;) {
+    const uint64_t h = (uint64_t)lo + step;
+    if (h >= e) {
+      hi = e;
+      break;
+    }
+    if ((int64_t)ld_stream_w(&adj[h]) >= t) {
+      hi = (uint32_t)h;
+      break;
+    }
+    lo = (uint32_t)h;
+    step <<= 1;
+  }
+  return lower_bound_w(adj, lo + 1, hi, t);
+}
+
 struct RoundCtx {
   int64_t lb, ub, ub_eff, st, lb0;
   uint32_t rid;
@@ -545,7 +575,7 @@ __device__ void round_phase(const KArgs& A, const RoundCtx& R, const Local& L, R
           const int64_t hi = R.ub_eff - (int64_t)d;
           if (hi > 0) {
             b = lower_bound_w(A.G.adj, rb, re, R.lb - (int64_t)d);
-            const uint32_t e = gallop_w(A.G.adj, b, re, hi);
+            const uint32_t e = gallop4_w(A.G.adj, b, re, hi);
             if (re - rb > kCursorMin) __stcg(&A.cursor[u], e - rb);
             len = e - b;
           }
@@ -561,8 +591,8 @@ __device__ void round_phase(const KArgs& A, const RoundCtx& R, const Local& L, R
             const uint32_t cur = rec.w;
             // windows of consecutive steps are contiguous: resume at the cursor
             b = cur == kNone ? lower_bound_w(A.G.adj, rb, re, R.lb - (int64_t)d)
-                             : gallop_w(A.G.adj, rb + cur, re, R.lb - (int64_t)d);
-            const uint32_t e = gallop_w(A.G.adj, b, re, R.ub_eff - (int64_t)d);
+                             : gallop4_w(A.G.adj, rb + cur, re, R.lb - (int64_t)d);
+            const uint32_t e = gallop4_w(A.G.adj, b, re, R.ub_eff - (int64_t)d);
             __stcg(&A.scur[idx], e - rb);
             len = e - b;
           }
@@ -601,7 +631,7 @@ __device__ void round_phase(const KArgs& A, const RoundCtx& R, const Local& L, R
           if (plong) {  // the prefix goes on past the lane's entries: find its end, then the rest
                         // is a window like a push window (the warp's concatenation, or grid tasks)
             b = z.z + kPullFast;
-            const uint32_t e = pull_bound > (int64_t)A.G.maxw ? z.w : gallop_w(A.G.adj, b, z.w, pull_bound);
+            const uint32_t e = pull_bound > (int64_t)A.G.maxw ? z.w : gallop4_w(A.G.adj, b, z.w, pull_bound);
             len = e - b;
           }
         }
