@@ -121,7 +121,7 @@ struct Workspace {
   uint32_t ring_bits = 0, ring_shift = 0;
   uint32_t task_cap = 0, step_cap = 0;
   uint64_t bytes = 0;
-  int grid = 0, block = 0;  // cached cooperative launch shape of k_eic
+  int grid = 0, block = 0, sms = 0;  // co-resident blocks of k_eic at this block size, and the SMs
 };
 
 struct eic_graph {

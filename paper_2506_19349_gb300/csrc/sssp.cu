@@ -2596,6 +2596,21 @@ struct DeviceGuard {
   ~DeviceGuard() { cudaSetDevice(prev); }
 };
 
+// Blocks a query runs on, of the sms * per_sm that fit: all of them, or 512
+// threads on every SM for a query that is a chain of small steps, where a
+// second block on the SM only slows the first one's chain (whether 152, 76 or 38
+// blocks remain makes no difference to such a query). Measured with 304 and
+// 152 blocks: RMAT 4 k 441, 376 us; 250 k 593, 564; 1 M vertices (650 k not
+// isolated) 698, 672; 2 M 806, 804; 4 M 957, 1034; uniform 16 k 399, 368; 131 k
+// 506, 509; 1 M 813, 841; grids 1024^2 24.1, 23.1 ms; 2048^2 46.9, 44.6; at
+// gap_shift 4 1000^2 4.95, 4.80, 3000^2 15.6, 15.8.
+int query_blocks(const DevGraph& G, const eic_params& p, int block, int sms, int per_sm) {
+  const uint64_t vertices = (uint64_t)G.ni << p.gap_shift;  // (wider steps settle more at a time)
+  const uint64_t most = fuse_items(G, p.heavy_min, p.flags) == kFuseRoad ? 1ull << 26 : 3ull << 18;
+  if (vertices > most) return sms * per_sm;
+  return sms * std::min(per_sm, std::max(1, kDefaultBlock / block));
+}
+
 // The cooperative grid of the query kernel, cached per workspace for the block
 // size last used.
 int launch_shape(Workspace* ws, int block) {
@@ -2609,6 +2624,7 @@ int launch_shape(Workspace* ws, int block) {
   EIC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wide ? k_eic<true> : k_eic<false>, block, 0));
   if (per_sm < 1) return EIC_ECUDA;
   ws->grid = sms * per_sm;
+  ws->sms = sms;
   ws->block = block;
   return EIC_OK;
 }
@@ -2670,7 +2686,7 @@ int enqueue_query(eic_graph* g, uint32_t s, uint32_t* dist, uint32_t* parent, co
   const int block = p.block_threads ? (int)p.block_threads : kDefaultBlock;
   int rc = launch_shape(&w, block);
   if (rc) return rc;
-  const int grid = w.grid;
+  const int grid = query_blocks(g->dg, p, block, w.sms, w.grid / w.sms);
   KArgs A = make_args(g, s, dist, p, status_out, grid);
   if (timeline) {
     A.timeline = w.timeline;
@@ -2683,7 +2699,7 @@ int enqueue_query(eic_graph* g, uint32_t s, uint32_t* dist, uint32_t* parent, co
   EIC_CUDA_TRY(cudaLaunchCooperativeKernel(w.ring_shift ? (const void*)k_eic<true> : (const void*)k_eic<false>, dim3(grid),
                                            dim3(block), args, 0, st));
   if (ev1) EIC_CUDA_TRY(cudaEventRecord(ev1, st));
-  k_output<<<4 * grid, 256, 0, st>>>(g->dg, w.idist, s, dist);
+  k_output<<<4 * w.grid, 256, 0, st>>>(g->dg, w.idist, s, dist);
   EIC_CUDA_TRY(cudaGetLastError());
   if (parent) {
     k_parent<<<1024, 256, 0, st>>>(g->dg, w.idist, s, parent);
@@ -3440,7 +3456,7 @@ static __device__ __align__(256) unsigned char g_na_scratch[kNaBytes];
 struct NaDevice {
   bool ready = false;
   unsigned char* base = nullptr;  // device address of g_na_scratch on this device
-  int grid = 0;
+  int grid = 0, sms = 0;
 };
 NaDevice g_na[kMaxDevices];
 std::mutex g_na_mu;
@@ -3464,6 +3480,7 @@ int na_setup(NaDevice& d, cudaStream_t st) {
   EIC_CUDA_TRY(cudaStreamSynchronize(st));
   d.base = base;
   d.grid = sms * per_sm;
+  d.sms = sms;
   d.ready = true;
   return EIC_OK;
 }
@@ -3527,15 +3544,19 @@ extern "C" int eic_sssp_noalloc(const eic_graph* gc, uint32_t source, uint32_t* 
   A.trace_cap = 0;
   A.timeline = nullptr;
   A.timeline_cap = 0;
-  A.nb = (uint32_t)nd.grid;
   A.fuse = fuse_items(G, A.heavy_min, A.flags);
+  eic_params p;
+  eic_params_default(&p);
+  p.heavy_min = A.heavy_min;
+  const int grid = query_blocks(G, p, kDefaultBlock, nd.sms, nd.grid / nd.sms);
+  A.nb = (uint32_t)grid;
   // Once anything is enqueued, every return waits for the stream first: the
   // next call may reuse the scratch only when this call's work has finished.
   auto enqueue = [&]() -> int {
     k_init<<<init_grid(A), 256, 0, st>>>(A);
     EIC_CUDA_TRY(cudaGetLastError());
     void* args[] = {&A};
-    EIC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_eic<false>, dim3(nd.grid), dim3(kDefaultBlock), args, 0, st));
+    EIC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_eic<false>, dim3(grid), dim3(kDefaultBlock), args, 0, st));
     k_output<<<4 * nd.grid, 256, 0, st>>>(G, A.dist, source, dist);
     EIC_CUDA_TRY(cudaGetLastError());
     return EIC_OK;
