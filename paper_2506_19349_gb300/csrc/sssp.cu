@@ -92,6 +92,7 @@ struct KArgs {
   unsigned long long* timeline;  // NULL unless the caller asked for it
   uint32_t timeline_cap;
   uint32_t nb;  // blocks working on this query: the grid, or one block group of a batch
+  uint32_t sweep_words;  // see sweep_chunk
   uint32_t fuse;  // rounds of at most this many items per warp are fused (see fuse_items; 0: none)
 };
 
@@ -107,7 +108,14 @@ constexpr uint32_t kTaskLen = 64;     // adjacency entries per grid task
 constexpr uint32_t kPullFastSingle = 8, kRelaxIlpSingle = 2;  // k_eic
 constexpr uint32_t kPullFastGroup = 4, kRelaxIlpGroup = 1;    // k_eic_batch, k_eic_serve
 constexpr uint32_t kSweepNum = 1, kSweepDen = 2;  // sweep the pull set when it holds >= 1/2 of the vertices
-constexpr uint32_t kSweepChunk = 16;  // settled-bitmap words a warp takes at a time in a sweep (<= 32)
+// Settled-bitmap words a warp takes at a time in a sweep: 16 (512 vertices, at
+// most 32 words), or fewer on a small graph so that every warp gets four
+// chunks: with 16, 90 k vertices kept 178 of 4864 warps busy for 16 batches each.
+constexpr uint32_t kSweepChunk = 16;
+__host__ __device__ inline uint32_t sweep_chunk(uint32_t ni, uint32_t blocks, uint32_t block_threads) {
+  const uint32_t w = (ni / 32 + 1) / (4 * blocks * (block_threads / 32));
+  return w < 1 ? 1 : w < kSweepChunk ? w : kSweepChunk;
+}
 constexpr uint32_t kStageT = 1024;    // tasks staged per block
 constexpr uint32_t kWarpStage = 256;  // next-frontier / settled-list appends staged per warp
 
@@ -528,7 +536,10 @@ __device__ void round_phase(const KArgs& A, const RoundCtx& R, const Local& L, R
   const bool sweep = round1 && L.pull_sweep;  // the pull set is every unsettled vertex, swept below
   const uint32_t npp = np + (sweep ? 0u : L.pull_cnt);
   const uint32_t nlisted = sweep ? nitems - L.pull_cnt : nitems;  // items of the listed part
-  const uint32_t gwarp = qblock(A) * (nt >> 5) + warp, nwarps = A.nb * (nt >> 5);
+  const uint32_t nwarps = A.nb * (nt >> 5);
+  // items a warp takes at a time: 32, or fewer so that a small round reaches every warp, the blocks in turn
+  const uint32_t per = nlisted >= 32 * nwarps ? 32u : max(1u, (nlisted + nwarps - 1) / nwarps);
+  const uint32_t gwarp = per == 32 ? qblock(A) * (nt >> 5) + warp : warp * A.nb + qblock(A);
   const int64_t pull_bound = R.ub - R.st;
   WarpScr& W = S.w[warp];
   WarpList Qw = {T.wq[warp], 0u, R.qcnt_out, R.qout};
@@ -738,14 +749,15 @@ __device__ void round_phase(const KArgs& A, const RoundCtx& R, const Local& L, R
     on_claimed(A, R, pok, psap, u, pbest, pold, C, Qw, Fw);
     __syncwarp();
   };
-  const uint32_t stride = nwarps * 32;
-  uint4 pre = fetch(gwarp * 32 + lane, fetch_id(gwarp * 32 + lane));
-  uint32_t idn = fetch_id(gwarp * 32 + stride + lane);
-  for (uint32_t base = gwarp * 32; base < nlisted; base += stride) {
-    const uint32_t i = base + lane;
+  const uint32_t stride = nwarps * per;
+  auto item = [&](uint32_t base) -> uint32_t { return lane < per ? base + lane : kNone; };
+  uint4 pre = fetch(item(gwarp * per), fetch_id(item(gwarp * per)));
+  uint32_t idn = fetch_id(item(gwarp * per + stride));
+  for (uint32_t base = gwarp * per; base < nlisted; base += stride) {
+    const uint32_t i = item(base);
     const uint4 rec = pre;
-    pre = fetch(base + stride + lane, idn);
-    idn = fetch_id(base + 2 * stride + lane);
+    pre = fetch(item(base + stride), idn);
+    idn = fetch_id(item(base + 2 * stride));
     step_items(rec, i, i >= nlisted ? kKindNone : (!round1 || i >= npp) ? kKindVertex : i < np ? kKindPush : kKindPull);
   }
   if (sweep) {
@@ -753,15 +765,15 @@ __device__ void round_phase(const KArgs& A, const RoundCtx& R, const Local& L, R
     // kSweepChunk settled-bitmap words (32 vertices each) at a time and hands
     // its lanes only the unsettled vertices, 32 per iteration, the next
     // batch's row bounds loaded while the current one runs
-    const uint32_t ni = A.G.ni, nwords = (ni + 31) >> 5, nchunks = (nwords + kSweepChunk - 1) / kSweepChunk;
+    const uint32_t ni = A.G.ni, nwords = (ni + 31) >> 5, nchunks = (nwords + A.sweep_words - 1) / A.sweep_words;
     uint32_t ch = gwarp, m = 0, off = 0, tot = 0, r0 = 0, wn = ~0u;
     auto word_at = [&](uint32_t c) -> uint32_t {
-      const uint32_t wi = c * kSweepChunk + lane;
-      return c < nchunks && lane < kSweepChunk && wi < nwords ? __ldcg(&A.sbits[wi]) : ~0u;
+      const uint32_t wi = c * A.sweep_words + lane;
+      return c < nchunks && lane < A.sweep_words && wi < nwords ? __ldcg(&A.sbits[wi]) : ~0u;
     };
     auto open_chunk = [&](uint32_t word) {  // this lane's unsettled mask, its exclusive rank, the chunk total
-      const uint32_t wi = ch * kSweepChunk + lane;
-      uint32_t mm = lane < kSweepChunk && wi < nwords ? ~word : 0u;
+      const uint32_t wi = ch * A.sweep_words + lane;
+      uint32_t mm = lane < A.sweep_words && wi < nwords ? ~word : 0u;
       if (wi == nwords - 1 && (ni & 31u)) mm &= (1u << (ni & 31u)) - 1u;
       m = mm;
       const uint32_t c = __popc(mm), inc = warp_incl_scan(c);
@@ -793,7 +805,7 @@ __device__ void round_phase(const KArgs& A, const RoundCtx& R, const Local& L, R
       const uint32_t ml = __shfl_sync(EIC_FULL_MASK, m, l), ol = __shfl_sync(EIC_FULL_MASK, off, l);
       if (r >= tot) return make_uint4(0u, 0u, 0u, 0u);
       ok = true;
-      const uint32_t v = ((ch * kSweepChunk + l) << 5) + kth_set_bit(ml, r - ol);
+      const uint32_t v = ((ch * A.sweep_words + l) << 5) + kth_set_bit(ml, r - ol);
       const uint2 rr = row_of(A.G, v);
       return make_uint4(v, 0u, rr.x, rr.x + rr.y);  // {vertex, settled word 0, row}
     };
@@ -2312,6 +2324,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_batch(BatchArgs P) {
       sA.timeline_cap = 0;
       sA.nb = P.nb;
       sA.fuse = bq.fuse;
+      sA.sweep_words = sweep_chunk(bq.G.ni, P.nb, blockDim.x);
     }
     __syncthreads();
     if (!query_setup(sA, ticket)) break;
@@ -2498,6 +2511,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_serve(ServeArgs P) {
       sA.timeline_cap = 0;
       sA.nb = P.nb;
       sA.fuse = bq.fuse;
+      sA.sweep_words = sweep_chunk(bq.G.ni, P.nb, blockDim.x);
     }
     __syncthreads();
     if (!query_setup(sA, ticket)) break;
@@ -2667,6 +2681,7 @@ KArgs make_args(eic_graph* g, uint32_t s, uint32_t* dist, const eic_params& p, i
   A.timeline_cap = 0;
   A.nb = (uint32_t)grid;
   A.fuse = fuse_items(g->dg, p.heavy_min, p.flags);
+  A.sweep_words = sweep_chunk(g->dg.ni, (uint32_t)grid, p.block_threads ? p.block_threads : kDefaultBlock);
   return A;
 }
 
@@ -3541,6 +3556,7 @@ extern "C" int eic_sssp_noalloc(const eic_graph* gc, uint32_t source, uint32_t* 
   p.heavy_min = A.heavy_min;
   const int grid = query_blocks(G, p, kDefaultBlock, nd.sms, nd.grid / nd.sms);
   A.nb = (uint32_t)grid;
+  A.sweep_words = sweep_chunk(G.ni, (uint32_t)grid, kDefaultBlock);
   // Once anything is enqueued, every return waits for the stream first: the
   // next call may reuse the scratch only when this call's work has finished.
   auto enqueue = [&]() -> int {
