@@ -23,6 +23,7 @@
 // Read-only view of a device-resident graph (preprocessing of Section 4.1).
 // Vertices have internal ids 0..ni-1: the non-isolated vertices ordered by
 // (degree descending, original id); orig2int/int2orig translate.
+constexpr uint32_t kBigRow = 512;    // longer rows are shared out when parents are looked for
 constexpr uint32_t kCursorMin = 16;  // rows longer than this keep a window cursor
 
 struct DevGraph {
@@ -47,6 +48,7 @@ struct DevGraph {
   const uint32_t* nz_lt;  // [nz_lt_len] nz_lt[t] = number of nz entries with smallest weight < t
   uint32_t nz_lt_len;
   uint32_t maxw, minw, max_deg, highd0;
+  uint32_t nbig, big_end;  // internal vertices of degree > kBigRow: ids [0, nbig), entries [0, big_end)
   uint32_t nlong;         // internal vertices of degree > kCursorMin: ids [0, nlong), the rows with a window cursor
 };
 

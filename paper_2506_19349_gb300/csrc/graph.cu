@@ -644,7 +644,7 @@ int build(eic_graph* g, const uint32_t* src, const uint32_t* dst, const uint32_t
 
   // 5b. distinct-degree tables and highD(0)
   const uint32_t hlen = maxdeg + 1;
-  uint32_t D = 0, nlong = 0;
+  uint32_t D = 0, nlong = 0, nbig = 0, big_end = 0;
   {
     uint64_t* pos;
     TRY(tmp.alloc(&pos, 2 * ((uint64_t)hlen + 1)));
@@ -680,6 +680,10 @@ int build(eic_graph* g, const uint32_t* src, const uint32_t* dst, const uint32_t
         acc += cnt[r];
         off += (uint64_t)cnt[r] * vals[r];
         if (vals[r] > kCursorMin) nlong = (uint32_t)acc;  // ids [0, acc) have degree >= vals[r]
+        if (vals[r] > kBigRow) {
+          nbig = (uint32_t)acc;
+          big_end = (uint32_t)off;
+        }
       }
       EIC_CUDA_TRY(cudaMemcpyAsync(g->dfirst, first.data(), (uint64_t)D * 4, cudaMemcpyHostToDevice, st));
       EIC_CUDA_TRY(cudaMemcpyAsync(g->drow, rows.data(), (uint64_t)D * sizeof(uint4), cudaMemcpyHostToDevice, st));
@@ -757,6 +761,8 @@ int build(eic_graph* g, const uint32_t* src, const uint32_t* dst, const uint32_t
   dg.dhint = g->dhint;
   dg.drow = g->drow;
   dg.nlong = nlong;
+  dg.nbig = nbig;
+  dg.big_end = big_end;
   dg.D = D;
   dg.rtow = g->rtow;
   dg.nz = g->nz;

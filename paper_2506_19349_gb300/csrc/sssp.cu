@@ -2201,29 +2201,66 @@ __global__ void k_output(DevGraph G, const uint32_t* __restrict__ idist, uint32_
   }
 }
 
-// parent[v] = smallest original id u with dist[u] + w(u, v) == dist[v] (one
-// warp per vertex); parent[s] = s, +inf where unreachable.
-__global__ void k_parent(DevGraph G, const uint32_t* __restrict__ idist, uint32_t s, uint32_t* parent) {
-  const uint32_t lane = lane_id();
-  const uint64_t nw = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  for (uint64_t v = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); v < G.n; v += nw) {
-    const uint32_t vi = G.orig2int[v];
-    const uint32_t dv = vi == EIC_INF ? EIC_INF : idist[vi];
+// parent[v] = smallest original id u with dist[u] + w(u, v) == dist[v]; parent[s]
+// = s, +inf where unreachable. Bound by the chain id -> distance -> entries ->
+// their distances of every vertex, and by the longest row: eight lanes take a
+// row (a warp's 32 mostly idled), and rows of more than kBigRow entries, which
+// come first in the adjacency, are shared out over the grid by k_parent_big.
+// With parents a query of an RMAT graph of 250 k vertices (longest row 24 k)
+// takes 52 us longer (159 before), of 2^22 402 us (652), of 2^25 4.4 ms (9.1).
+constexpr uint32_t kParentLanes = 8;
+constexpr uint32_t kBigChunk = 256;  // entries of the big rows a warp takes at a time
+
+// best[vi] (all ones before): the parent of the vertices with big rows.
+__global__ void k_parent_big(DevGraph G, const uint32_t* __restrict__ idist, uint32_t* best) {
+  const uint32_t lane = lane_id(), wpb = blockDim.x >> 5;
+  const uint64_t nw = (uint64_t)gridDim.x * wpb;
+  for (uint64_t at = ((uint64_t)blockIdx.x * wpb + (threadIdx.x >> 5)) * kBigChunk; at < G.big_end; at += nw * kBigChunk) {
+    uint32_t lo = 0, hi = G.nbig - 1;  // the row that holds the chunk's first entry
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (__ldg(&G.row[mid]) <= at)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    const uint64_t end = min(at + kBigChunk, (uint64_t)G.big_end);
+    uint32_t vi = lo, re = __ldg(&G.row[lo + 1]);
+    for (uint64_t i = at + lane; i < end; i += 32) {
+      while (i >= re) re = __ldg(&G.row[++vi + 1]);
+      const uint32_t dv = __ldg(&idist[vi]);
+      const uint2 ent = __ldg(&G.adj[i]);
+      if (dv == EIC_INF || ent.y > dv) continue;
+      const uint32_t du = __ldg(&idist[ent.x]);
+      if (du != EIC_INF && (uint64_t)du + ent.y == dv) atomicMin(&best[vi], __ldg(&G.int2orig[ent.x]));
+    }
+  }
+}
+
+__global__ void k_parent(DevGraph G, const uint32_t* __restrict__ idist, const uint32_t* __restrict__ big, uint32_t s,
+                         uint32_t* parent) {
+  const uint32_t sub = threadIdx.x % kParentLanes;
+  const uint32_t mask = ((1u << kParentLanes) - 1u) << (lane_id() - sub);
+  const uint64_t step = (uint64_t)gridDim.x * (blockDim.x / kParentLanes);
+  for (uint64_t v = (uint64_t)blockIdx.x * (blockDim.x / kParentLanes) + threadIdx.x / kParentLanes; v < G.n; v += step) {
+    const uint32_t vi = __ldg(&G.orig2int[v]);
     uint32_t best = EIC_INF;
-    if (v != s && dv != EIC_INF) {
-      const uint32_t rb = G.row[vi], re = G.row[vi + 1];
-      for (uint32_t i = rb + lane; i < re; i += 32) {
-        const uint2 ent = G.adj[i];
-        if (ent.y > dv) break;
-        const uint32_t du = idist[ent.x];
-        if (du != EIC_INF && (uint64_t)du + ent.y == dv) {
-          const uint32_t uo = G.int2orig[ent.x];
-          best = uo < best ? uo : best;
+    if (vi != EIC_INF && v != s) {
+      if (vi < G.nbig) {
+        best = __ldg(&big[vi]);
+      } else {
+        const uint32_t dv = __ldg(&idist[vi]);
+        const uint2 rr = dv != EIC_INF ? row_of(G, vi) : make_uint2(0u, 0u);
+        for (uint32_t i = rr.x + sub; i < rr.x + rr.y; i += kParentLanes) {
+          const uint2 ent = __ldg(&G.adj[i]);
+          if (ent.y > dv) break;  // (rows are in weight order)
+          const uint32_t du = __ldg(&idist[ent.x]);
+          if (du != EIC_INF && (uint64_t)du + ent.y == dv) best = min(best, __ldg(&G.int2orig[ent.x]));
         }
       }
-      for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(EIC_FULL_MASK, best, o));
     }
-    if (lane == 0) parent[v] = v == s ? s : best;
+    best = __reduce_min_sync(mask, best);
+    if (sub == 0) parent[v] = v == s ? s : best;
   }
 }
 
@@ -2713,7 +2750,13 @@ int enqueue_query(eic_graph* g, uint32_t s, uint32_t* dist, uint32_t* parent, co
   k_output<<<4 * w.grid, 256, 0, st>>>(g->dg, w.idist, s, dist);
   EIC_CUDA_TRY(cudaGetLastError());
   if (parent) {
-    k_parent<<<1024, 256, 0, st>>>(g->dg, w.idist, s, parent);
+    if (g->dg.nbig) {  // (the queue's words have served)
+      EIC_CUDA_TRY(cudaMemsetAsync(w.q[0], 0xFF, (uint64_t)g->dg.nbig * 4, st));
+      k_parent_big<<<(unsigned)std::min<uint64_t>(8 * w.sms, g->dg.big_end / (8 * kBigChunk) + 1), 256, 0, st>>>(
+          g->dg, w.idist, w.q[0]);
+    }
+    k_parent<<<(unsigned)std::min<uint64_t>(8 * w.sms, (uint64_t)g->dg.n / 32 + 1), 256, 0, st>>>(g->dg, w.idist, w.q[0],
+                                                                                                  s, parent);
     EIC_CUDA_TRY(cudaGetLastError());
   }
   return EIC_OK;
