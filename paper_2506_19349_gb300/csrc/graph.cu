@@ -18,7 +18,7 @@
 // sorting passes over the pairs and four over the entries, each reading a key
 // twice and writing it once, with the weight (and neighbour) inside the key. A
 // build took 25.7 ms before (12-byte pairs in seven passes, one atomic per
-// degree, a one-block scan per pass) and takes 6.5 ms, of which the sorts are
+// degree, a one-block scan per pass) and takes 6.4 ms, of which the sorts are
 // 3.2 and allocation 1.9.
 #include <stdlib.h>
 #include <string.h>
@@ -232,10 +232,15 @@ __global__ void __launch_bounds__(kThreads) k_emit(const uint64_t* __restrict__ 
 
 // First entry and end of every row of the sorted entries (row = key >> lo; zero where a vertex has none).
 __global__ void k_row_ends(const uint64_t* __restrict__ keys, uint64_t E, int lo, uint32_t* beg, uint32_t* end) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < E; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t r = keys[i] >> lo;
-    if (i == 0 || (keys[i - 1] >> lo) != r) beg[r] = (uint32_t)i;
-    if (i + 1 == E || (keys[i + 1] >> lo) != r) end[r] = (uint32_t)(i + 1);
+  const uint32_t lane = threadIdx.x & 31u;  // (a lane's neighbours hold the entries beside its own)
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i - lane < E; i += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t none = ~0ull, r = i < E ? keys[i] >> lo : none;
+    uint64_t before = __shfl_up_sync(EIC_FULL_MASK, r, 1), after = __shfl_down_sync(EIC_FULL_MASK, r, 1);
+    if (lane == 0) before = i > 0 && i < E ? keys[i - 1] >> lo : none;
+    if (lane == 31) after = i + 1 < E ? keys[i + 1] >> lo : none;
+    if (i >= E) continue;
+    if (before != r) beg[r] = (uint32_t)i;
+    if (after != r) end[r] = (uint32_t)(i + 1);
   }
 }
 
@@ -251,16 +256,24 @@ __global__ void k_row_lengths(const uint32_t* __restrict__ beg, uint32_t* end, u
   if ((threadIdx.x & 31) == 0 && lmax) atomicMax(maxdeg, lmax);
 }
 
+// beg[v] to what a row's entries move by (modulo 2^32): its place in internal order minus its first entry.
+__global__ void k_row_shift(uint32_t* beg, uint64_t n, const uint32_t* __restrict__ orig2int,
+                            const uint32_t* __restrict__ row) {
+  for (uint64_t v = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v < n; v += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t i = orig2int[v];
+    if (i != 0xFFFFFFFFu) beg[v] = row[i] - beg[v];
+  }
+}
+
 // The sorted entries to their places: rows in internal order, neighbours renamed.
 template <bool kVals>
 __global__ void k_place(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals, uint64_t E, int vbits,
-                        int wb, const uint32_t* __restrict__ beg, const uint32_t* __restrict__ orig2int,
-                        const uint32_t* __restrict__ row, uint2* adj) {
+                        int wb, const uint32_t* __restrict__ shift, const uint32_t* __restrict__ orig2int, uint2* adj) {
   const uint64_t vmask = (1ull << vbits) - 1, wmask = (1ull << wb) - 1;
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < E; i += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t k = keys[i], rw = kVals ? k : k >> vbits;
     const uint32_t v = kVals ? vals[i] : (uint32_t)(k & vmask), u = (uint32_t)(rw >> wb);
-    adj[row[orig2int[u]] + ((uint32_t)i - beg[u])] = make_uint2(orig2int[v], (uint32_t)(rw & wmask));
+    adj[(uint32_t)i + shift[u]] = make_uint2(orig2int[v], (uint32_t)(rw & wmask));
   }
 }
 
@@ -621,10 +634,11 @@ int build(eic_graph* g, const uint32_t* src, const uint32_t* dst, const uint32_t
   }
   TRY(galloc(g, &g->adj, E + 2));  // two spare entries: a 16-byte pair load starting at the last entry stays inside
   if (E > 0) {
+    k_row_shift<<<grid_for(n), kThreads, 0, st>>>(beg, n, g->orig2int, g->row);
     if (packed)
-      k_place<false><<<grid_for(E), kThreads, 0, st>>>(ka, nullptr, E, vbits, wb, beg, g->orig2int, g->row, g->adj);
+      k_place<false><<<grid_for(E), kThreads, 0, st>>>(ka, nullptr, E, vbits, wb, beg, g->orig2int, g->adj);
     else
-      k_place<true><<<grid_for(E), kThreads, 0, st>>>(ka, va, E, vbits, wb, beg, g->orig2int, g->row, g->adj);
+      k_place<true><<<grid_for(E), kThreads, 0, st>>>(ka, va, E, vbits, wb, beg, g->orig2int, g->adj);
     EIC_CUDA_TRY(cudaGetLastError());
   }
 

@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_radix_scatter(const uint64_
       uint32_t peers = __ballot_sync(EIC_FULL_MASK, in);
 #pragma unroll
       for (int b = 0; b < kRadixBits; ++b) {
+        if (!((mask >> b) & 1u)) break;  // (the pass's digits are narrower)
         const uint32_t m = __ballot_sync(EIC_FULL_MASK, (d >> b) & 1u);
         peers &= (d >> b) & 1u ? m : ~m;
       }
