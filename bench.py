@@ -77,7 +77,7 @@ KERNEL_SOURCES = ("paper_2506_19349_gb300/csrc/sssp.cu", "paper_2506_19349_gb300
                   "paper_2506_19349_gb300/csrc/graph.h", "paper_2506_19349_gb300/csrc/graph.cu",
                   "paper_2506_19349_gb300/csrc/stats.cuh", "include/eic.h")
 MEASURED_TRAFFIC = {  # {(scale, kernel code sha256): bytes per launch}
-    (25, "298c3629a5385ee6ab3745012138720b3479de107e64f161049f176bd47c3fcd"): 6088278784,
+    (25, "30648cf05254c4de797f22ccc62c9fe0934d95a6fdb8918cb8aa888cc4c488c9"): 4848897728,
 }
 
 

@@ -313,7 +313,8 @@ int eic_batch_destroy(eic_batch* b);
  * while there is work: after config.idle_us without a request, once no
  * request runs, a block group registers as idle, and when every group is
  * registered they leave together; the runtime relaunches the kernel when
- * requests arrive again. The width of a launch follows the backlog: with at
+ * requests arrive again. A launch waits until no request has come for 12 us
+ * (at most 250 us), so that a burst is seen whole. The width of a launch follows the backlog: with at
  * most 4 (8, 16) waiting requests it runs 4 (8, 16) groups that share the
  * co-resident blocks, else config.groups groups; a launch with fewer groups
  * ends (each group after its current request) once twice its group count of

@@ -27,13 +27,15 @@
 // Phases (one grid barrier each): a round (the first round of a step runs
 // Function 1's push set and pull), an optional task phase, and per step one
 // statistics pass after which block 0 evaluates Eq. 1-3 and Function 2 and
-// publishes the next <st, lb, ub>. In a round each warp takes 32 items at a
-// time (warp-strided, its next items' records loaded ahead); each lane finds
-// its item's window in the weight-sorted row, and the warp relaxes the
-// concatenation of its lanes' windows, windows longer than heavy_min becoming
-// 64-entry tasks for the task phase. A pull set of at least half the vertices
-// is swept in vertex order over the unsettled vertices only, compacted from
-// the settled bitmap 512 vertices at a time.
+// publishes the next <st, lb, ub> (with weights of 2^20 and above, after all
+// blocks have filled Function 2's bins). In a round each warp takes up to 32
+// items at a time (warp-strided, its next items' records loaded ahead); each
+// lane finds its item's window in the weight-sorted row, and the warp relaxes
+// the concatenation of its lanes' windows, windows longer than heavy_min
+// becoming 64-entry tasks for the task phase. A pull set of at least half the
+// vertices is swept in vertex order over the unsettled vertices only,
+// compacted from the settled bitmap up to 512 vertices at a time. A round with
+// few items is fused with those that follow it in the step (fused_round).
 #include <stdlib.h>
 #include <string.h>
 
