@@ -75,7 +75,7 @@ def dist_env():
 # their comments and blank lines, and any change to the code reports null.
 KERNEL_SOURCES = ("paper_2506_19349_gb300/csrc/sssp.cu", "paper_2506_19349_gb300/csrc/common.cuh",
                   "paper_2506_19349_gb300/csrc/graph.h", "paper_2506_19349_gb300/csrc/graph.cu",
-                  "paper_2506_19349_gb300/csrc/stats.cuh", "include/eic.h")
+                  "paper_2506_19349_gb300/csrc/search.h", "paper_2506_19349_gb300/csrc/stats.cuh", "include/eic.h")
 MEASURED_TRAFFIC = {  # {(scale, kernel code sha256): bytes per launch}
     (25, "30648cf05254c4de797f22ccc62c9fe0934d95a6fdb8918cb8aa888cc4c488c9"): 4848897728,
 }

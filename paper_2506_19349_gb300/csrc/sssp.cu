@@ -44,6 +44,7 @@
 
 #include "graph.h"
 #include "pool.h"
+#include "search.h"
 #include "serve.h"
 #include "stats.cuh"
 
@@ -336,72 +337,22 @@ __device__ __forceinline__ uint4 ld_stream4(const uint4* p) {
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// first index in [b, e) of the weight-sorted row with weight >= t
-__device__ __forceinline__ uint32_t lower_bound_w(const uint2* __restrict__ adj, uint32_t b, uint32_t e, int64_t t) {
-  if (t <= 1) return b;  // weights are >= 1
-  while (b < e) {
-    uint32_t mid = b + ((e - b) >> 1);
-    if ((int64_t)ld_stream_w(&adj[mid]) < t)
-      b = mid + 1;
-    else
-      e = mid;
-  }
-  return b;
+// The window searches (search.h) over the adjacency's weights.
+struct AdjWeight {
+  const uint2* __restrict__ adj;
+  __device__ __forceinline__ uint32_t operator()(uint32_t i) const { return ld_stream_w(&adj[i]); }
+};
+
+__device__ __forceinline__ uint32_t lower_bound_w(const uint2* adj, uint32_t b, uint32_t e, int64_t t) {
+  return lower_bound(AdjWeight{adj}, b, e, t);
 }
 
-// The same, given that every entry before p has weight < t: exponential
-// probes forward from p, then a binary search in the last interval. Costs
-// O(log distance), and a short window costs one or two probes of one sector.
-__device__ __forceinline__ uint32_t gallop_w(const uint2* __restrict__ adj, uint32_t p, uint32_t e, int64_t t) {
-  if (t <= 1 || p >= e) return p;
-  if ((int64_t)ld_stream_w(&adj[p]) >= t) return p;
-  uint32_t lo = p;  // weight at lo < t
-  uint32_t hi;
-  uint64_t step = 1;
-  for (;;) {
-    const uint64_t h = (uint64_t)lo + step;
-    if (h >= e) {
-      hi = e;
-      break;
-    }
-    if ((int64_t)ld_stream_w(&adj[h]) >= t) {
-      hi = (uint32_t)h;
-      break;
-    }
-    lo = (uint32_t)h;
-    step <<= 1;
-  }
-  return lower_bound_w(adj, lo + 1, hi, t);
+__device__ __forceinline__ uint32_t gallop_w(const uint2* adj, uint32_t p, uint32_t e, int64_t t) {
+  return gallop(AdjWeight{adj}, p, e, t);
 }
 
-// The same for windows that mostly end within four entries: the weights of the
-// first four are read at once. (RMAT 2^25 2779 -> 2730 us, 15 M log-normal
-// 1885 -> 1863 us; a window's average length there is 1.3 entries.)
-__device__ __forceinline__ uint32_t gallop4_w(const uint2* __restrict__ adj, uint32_t p, uint32_t e, int64_t t) {
-  if (t <= 1 || p >= e) return p;
-  uint32_t w[4], c = 0;
-#pragma unroll
-  for (uint32_t k = 0; k < 4; ++k) w[k] = p + k < e ? ld_stream_w(&adj[p + k]) : 0xFFFFFFFFu;
-#pragma unroll
-  for (uint32_t k = 0; k < 4; ++k) c += p + k < e && (int64_t)w[k] < t ? 1u : 0u;
-  if (c < 4) return p + c;
-  uint32_t lo = p + 3;  // weight at lo < t
-  uint32_t hi;
-  uint64_t step = 1;
-  for (;;) {
-    const uint64_t h = (uint64_t)lo + step;
-    if (h >= e) {
-      hi = e;
-      break;
-    }
-    if ((int64_t)ld_stream_w(&adj[h]) >= t) {
-      hi = (uint32_t)h;
-      break;
-    }
-    lo = (uint32_t)h;
-    step <<= 1;
-  }
-  return lower_bound_w(adj, lo + 1, hi, t);
+__device__ __forceinline__ uint32_t gallop4_w(const uint2* adj, uint32_t p, uint32_t e, int64_t t) {
+  return gallop4(AdjWeight{adj}, p, e, t);
 }
 
 struct RoundCtx {
