@@ -102,13 +102,10 @@ struct SlotPool {
       s.step_ub = (int64_t*)(b + L.step_ub);
       s.step_off = (uint32_t*)(b + L.step_off);
       s.ctl = (Ctl*)(b + L.ctl);
-      if (cudaMemset(s.ctl, 0, sizeof(Ctl)) != cudaSuccess) {
-        (void)cudaGetLastError();
-        release();
-        return EIC_ECUDA;
-      }
     }
-    if (cudaMemcpy(d_slots, h.data(), sizeof(BatchSlot) * groups, cudaMemcpyHostToDevice) != cudaSuccess) {
+    // (a copy from pageable memory may return before it has arrived, and the launches that read it come on any stream)
+    if (cudaMemcpy(d_slots, h.data(), sizeof(BatchSlot) * groups, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaStreamSynchronize(nullptr) != cudaSuccess) {
       (void)cudaGetLastError();
       release();
       return EIC_ECUDA;

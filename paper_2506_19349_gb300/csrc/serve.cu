@@ -433,11 +433,13 @@ int eic_server_create(const eic_graph* const* graphs, uint32_t num_graphs, const
     memset(s->ring, 0, rbytes);
     s->ring->cap = s->cap;
   }
-  if (cudaMalloc((void**)&s->d_graphs, hq.size() * sizeof(BatchQuery)) != cudaSuccess ||
+  // (set up on the stream that the kernel is launched on: it does not wait for the legacy stream's work)
+  if (cudaStreamCreateWithFlags(&s->kstream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaMalloc((void**)&s->d_graphs, hq.size() * sizeof(BatchQuery)) != cudaSuccess ||
       cudaMalloc((void**)&s->d_claim, 4 * sizeof(unsigned long long)) != cudaSuccess ||
-      cudaMemcpy(s->d_graphs, hq.data(), hq.size() * sizeof(BatchQuery), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(s->d_claim, 0, 4 * sizeof(unsigned long long)) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&s->kstream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaMemcpyAsync(s->d_graphs, hq.data(), hq.size() * sizeof(BatchQuery), cudaMemcpyHostToDevice, s->kstream) !=
+          cudaSuccess ||
+      cudaMemsetAsync(s->d_claim, 0, 4 * sizeof(unsigned long long), s->kstream) != cudaSuccess ||
       cudaStreamCreateWithFlags(&s->cstream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->kdone, cudaEventDisableTiming) != cudaSuccess) {
     (void)cudaGetLastError();
@@ -606,8 +608,8 @@ int eic_server_tune(eic_server* s, const uint32_t* sample_sources, uint32_t* gap
     if (rc == EIC_OK) s->hq[k].gap_shift = best;
     if (gap_shifts) gap_shifts[k] = s->hq[k].gap_shift;
   }
-  if (rc == EIC_OK && cudaMemcpy(s->d_graphs, s->hq.data(), s->hq.size() * sizeof(BatchQuery),
-                                 cudaMemcpyHostToDevice) != cudaSuccess) {
+  if (rc == EIC_OK && cudaMemcpyAsync(s->d_graphs, s->hq.data(), s->hq.size() * sizeof(BatchQuery),
+                                      cudaMemcpyHostToDevice, s->kstream) != cudaSuccess) {
     (void)cudaGetLastError();
     rc = EIC_ECUDA;
   }

@@ -2820,11 +2820,6 @@ int eic_ws_ensure(eic_graph* g, int) {
     eic_ws_free(w);
     return EIC_ENOMEM;
   }
-  if (cudaMemset(w->ctl, 0, sizeof(Ctl)) != cudaSuccess) {
-    (void)cudaGetLastError();
-    eic_ws_free(w);
-    return EIC_ECUDA;
-  }
   return EIC_OK;
 }
 
@@ -3009,10 +3004,11 @@ int batch_configure(eic_batch* b, uint32_t groups, uint32_t block, uint32_t nb_f
   return EIC_OK;
 }
 
-// The host query table to the device (per-query parameters changed).
-int batch_upload(eic_batch* b) {
+// The host query table to the device (per-query parameters changed), before any later launch on any stream.
+int batch_upload(eic_batch* b, cudaStream_t st) {
   if (b->hq.empty()) return EIC_OK;
-  EIC_CUDA_TRY(cudaMemcpy(b->d_q, b->hq.data(), b->hq.size() * sizeof(BatchQuery), cudaMemcpyHostToDevice));
+  EIC_CUDA_TRY(cudaMemcpyAsync(b->d_q, b->hq.data(), b->hq.size() * sizeof(BatchQuery), cudaMemcpyHostToDevice, st));
+  EIC_CUDA_TRY(cudaStreamSynchronize(st));
   if (b->exec) {
     cudaGraphExecDestroy(b->exec);
     b->exec = nullptr;
@@ -3066,8 +3062,9 @@ void batch_free(eic_batch* b) {
   delete b;
 }
 
+// The query table is copied on st, which orders it before launches there.
 int batch_create(const eic_graph* const* graphs, const uint32_t* sources, uint32_t nq, uint32_t* const* dists,
-                 const eic_params* params, SlotPool* shared_pool, eic_batch** out) {
+                 const eic_params* params, SlotPool* shared_pool, cudaStream_t st, eic_batch** out) {
   *out = nullptr;
   if (nq == 0 || !graphs || !sources || !dists) return EIC_EINVAL;
   eic_params p;
@@ -3133,7 +3130,7 @@ int batch_create(const eic_graph* const* graphs, const uint32_t* sources, uint32
       batch_free(b);
       return EIC_ENOMEM;
     }
-    if (cudaMemcpy(b->d_q, b->hq.data(), nrun * sizeof(BatchQuery), cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (cudaMemcpyAsync(b->d_q, b->hq.data(), nrun * sizeof(BatchQuery), cudaMemcpyHostToDevice, st) != cudaSuccess) {
       (void)cudaGetLastError();
       batch_free(b);
       return EIC_ECUDA;
@@ -3220,14 +3217,14 @@ int eic_sssp_batch(const eic_graph* const* graphs, const uint32_t* sources, uint
   if (!guard.ok || graphs[0]->device < 0 || graphs[0]->device >= kMaxDevices) return EIC_ECUDA;
   std::lock_guard<std::mutex> lock(g_pool_mu);
   eic_batch* b = nullptr;
-  int rc = batch_create(graphs, sources, num_queries, dists, params, &g_pool[graphs[0]->device], &b);
+  cudaStream_t st = (cudaStream_t)stream;
+  int rc = batch_create(graphs, sources, num_queries, dists, params, &g_pool[graphs[0]->device], st, &b);
   if (rc) {
     if (statuses)
       for (uint32_t i = 0; i < num_queries; ++i) statuses[i] = rc;
     return rc;
   }
   b->use_graph = false;  // one-shot: launch directly
-  cudaStream_t st = (cudaStream_t)stream;
   rc = batch_enqueue(b, st);
   if (rc == EIC_OK) {
     rc = batch_wait(b, st, statuses);
@@ -3248,7 +3245,12 @@ int eic_batch_create(const eic_graph* const* graphs, const uint32_t* sources, ui
   if (!graphs || !graphs[0]) return EIC_EINVAL;
   DeviceGuard guard(graphs[0]->device);
   if (!guard.ok) return EIC_ECUDA;
-  return batch_create(graphs, sources, num_queries, dists, params, nullptr, out);
+  const int rc = batch_create(graphs, sources, num_queries, dists, params, nullptr, nullptr, out);
+  if (rc != EIC_OK || cudaStreamSynchronize(nullptr) == cudaSuccess) return rc;
+  (void)cudaGetLastError();
+  batch_free(*out);
+  *out = nullptr;
+  return EIC_ECUDA;
 }
 
 int eic_batch_run(eic_batch* b, void* stream) {
@@ -3283,7 +3285,7 @@ int eic_batch_tune(eic_batch* b, void* stream, eic_batch_config* best) {
         q.fuse = fuse_items(q.G, hm, b->p.flags);
       }
       b->p.heavy_min = hm;
-      int r = batch_upload(b);
+      int r = batch_upload(b, st);
       if (r) return r;
       if ((r = batch_configure(b, g, block))) return r;
       double ms = batch_time(b, st);
@@ -3337,14 +3339,14 @@ int eic_batch_tune(eic_batch* b, void* stream, eic_batch_config* best) {
         sd.push_back(b->qdist[j]);
       }
       eic_batch* sub = nullptr;
-      if ((rc = batch_create(sg.data(), ss.data(), (uint32_t)pos.size(), sd.data(), &b->p, nullptr, &sub)))
+      if ((rc = batch_create(sg.data(), ss.data(), (uint32_t)pos.size(), sd.data(), &b->p, nullptr, st, &sub)))
         return rc;
       rc = batch_configure(sub, (uint32_t)pos.size(), best_block, nb);
       uint32_t gs_best = b->hq[k].gap_shift;
       double t_best = -1.0;
       for (uint32_t gs = gs_best; rc == EIC_OK && gs <= 8; ++gs) {
         for (auto& q : sub->hq) q.gap_shift = gs;
-        if ((rc = batch_upload(sub))) break;
+        if ((rc = batch_upload(sub, st))) break;
         double t = batch_time(sub, st);
         const double t2 = batch_time(sub, st);
         if (t < 0 || t2 < 0) {
@@ -3378,7 +3380,7 @@ int eic_batch_tune(eic_batch* b, void* stream, eic_batch_config* best) {
       q.fuse = fuse_items(q.G, best_hm, b->p.flags);
     }
     b->p.heavy_min = best_hm;
-    if ((rc = batch_upload(b))) return rc;
+    if ((rc = batch_upload(b, st))) return rc;
     if (b->pool == &b->own && b->own.count > best_g) b->own.release();
     if ((rc = batch_configure(b, best_g, best_block))) return rc;
     if (b->exec) {
@@ -3621,12 +3623,12 @@ int eic_tune_step_width(const eic_graph* g, uint32_t source, uint32_t copies, ui
   std::vector<uint32_t*> ds;
   for (uint32_t k = 0; k < copies; ++k) ds.push_back(buf + n * k);
   eic_batch* b = nullptr;
-  int rc = batch_create(gs.data(), ss.data(), copies, ds.data(), &p, nullptr, &b);
+  int rc = batch_create(gs.data(), ss.data(), copies, ds.data(), &p, nullptr, stream, &b);
   if (rc == EIC_OK) rc = batch_configure(b, copies, p.block_threads ? p.block_threads : kDefaultBlock, nb);
   double t_best = -1.0;
   for (uint32_t shift = from; rc == EIC_OK && shift <= 8; ++shift) {
     for (auto& q : b->hq) q.gap_shift = shift;
-    if ((rc = batch_upload(b))) break;
+    if ((rc = batch_upload(b, stream))) break;
     double t = batch_time(b, stream);
     const double t2 = batch_time(b, stream);
     if (t < 0 || t2 < 0) {
