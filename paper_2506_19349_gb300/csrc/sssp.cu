@@ -151,6 +151,14 @@ constexpr uint32_t kFusePop = 8;      // queued vertices a warp takes at a time
 // and 32 iterations; windows of 64 and 256 entries differ by 2% either way.
 constexpr uint32_t kFuseLong = 64;
 constexpr uint32_t kFuseIters = 6;
+// Road-like graphs hand on after kRoadWaves waves (a step of a grid has some
+// tens), fewer where a wave may be long: it takes at most as many iterations as
+// the largest degree. The limit is for a chain that one group walks alone while
+// every other block waits at the barrier, whose wait is bounded (a path of 10^7
+// vertices in one step would outlast it): 1024 waves take 1.2 to 10 ms. The
+// group then queues nothing more, which costs the 4096^2 grid 0.1%; its queue
+// handed on as below cost 0.6%.
+constexpr uint32_t kRoadWaves = 1024, kRoadWavesMin = 64, kRoadIters = 8 * kRoadWaves;
 constexpr uint32_t kFuseQueue = 128 * kFuseWarps;  // entries of a local queue (a power of two)
 constexpr uint32_t kFuseGroups = (kMaxWarps + kFuseWarps - 1) / kFuseWarps;
 static_assert(kFuseGroups <= 15, "a group synchronises on named barrier 1 + its index; 0 is the block barrier");
@@ -1064,12 +1072,12 @@ __device__ __noinline__ int64_t block_st_bins(uint32_t* bins, uint32_t st_num, u
 // kRoad: no window is longer than heavy_min (every degree of the graph is at
 // most that). Otherwise a window may be too long for one warp: an item's then
 // becomes grid tasks, a vertex improved in the round waits for the next, plain
-// round; and a group that has spent kFuseIters iterations hands its queue to
-// the next round, where it is dealt to all warps again (34 items whose subtree
-// of 5000 vertices stayed in 34 groups took 220 us, plain rounds 130 us). On
-// such graphs it saves the 8 us of each small round: uniform 2^14 vertices 488
-// -> 394 us, RMAT 131 k 579 -> 518 us, RMAT 2^22 1029 -> 990 us, RMAT 2^25
-// 3.03 -> 2.94 ms a query.
+// round. A group that has spent its waves (kRoad) or kFuseIters iterations
+// leaves the rest to the next round, where it is dealt to all warps again (34
+// items whose subtree of 5000 vertices stayed in 34 groups took 220 us, plain
+// rounds 130 us). On graphs with long rows fusion saves the 8 us of each small
+// round: uniform 2^14 vertices 488 -> 394 us, RMAT 131 k 579 -> 518 us, RMAT
+// 2^22 1029 -> 990 us, RMAT 2^25 3.03 -> 2.94 ms a query.
 template <bool kRoad>
 __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, RoundScr& S, Stage& T,
                             uint32_t nitems, bool round1, const uint32_t* qin, Counters& C) {
@@ -1091,14 +1099,21 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
   const uint32_t np = round1 ? L.push_end - L.push_beg : 0;
   if (gw == 0 && lane < 3) fcnt[lane] = fstop[lane] = 0;
   group_sync();
-  uint32_t spent = 0;
+  uint32_t spent = 0;  // the warp's iterations
+  uint32_t waves = kRoad ? min(kRoadWaves, max(kRoadWavesMin, kRoadIters / A.G.max_deg)) : 0u;  // the group's waves left
   uint32_t lh = 0, lt = 0, wave = 0;  // the ring's head and tail, the wave mod 3 (the same in every thread of the group)
   while (i0 < i1 || lh != lt) {
     uint32_t d = EIC_INF, b = 0, len = 0, u = 0, rb = 0, deg = 0;
     uint32_t now = EIC_INF;  // a queued vertex's distance as its wave begins
     bool vertex = false;     // a frontier vertex (or the source): its window starts at its row
     bool seed = false;       // one of the round's items
-    const uint32_t room = kFuseQueue - (lt - lh);
+    uint32_t room = kFuseQueue - (lt - lh);
+    if (kRoad) {  // its waves spent, the group queues nothing more: what it improves goes to the next round
+      if (waves == 0)
+        room = 0;
+      else
+        --waves;
+    }
     if (i0 < i1) {
       const uint32_t take = min(i1 - i0, 32 * gn), each = (take + gn - 1) / gn;
       const uint32_t i = i0 + gw * each + lane;
