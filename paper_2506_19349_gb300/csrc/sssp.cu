@@ -1199,12 +1199,14 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, R
         __stcg(&R.qout[slot], u);
         __stcg(R.plain_out, 1u);
       }
+      if (lng && !seed) vertex = false;  // (relaxed, and counted, in the next round)
       if (lng) len = 0;
     }
     const uint32_t incl = warp_incl_scan(len);
     const uint32_t total = __shfl_sync(EIC_FULL_MASK, incl, 31);
     const uint32_t excl = incl - len, full = __ballot_sync(EIC_FULL_MASK, len != 0);  // lanes with a window
     uint32_t live = 0;  // lanes whose vertex still has the distance it was queued with
+    if (total == 0) C.frontier += vertex && now == d ? 1 : 0;
     if (!kRoad) {
       spent += (total + 31) / 32;
       if (spent > kFuseIters && lane == 0) fstop[wave] = 1;
