@@ -23,7 +23,7 @@
 // Read-only view of a device-resident graph (preprocessing of Section 4.1).
 // Vertices have internal ids 0..ni-1: the non-isolated vertices ordered by
 // (degree descending, original id); orig2int/int2orig translate.
-constexpr uint32_t kBigRow = 512;    // longer rows are shared out when parents are looked for
+constexpr uint32_t kBigRow = 256;    // a longer row is taken by a whole warp when parents are looked for
 constexpr uint32_t kCursorMin = 16;  // rows longer than this keep a window cursor
 
 struct DevGraph {

@@ -45,6 +45,7 @@ struct Ctl {
   uint32_t touched_cnt;
   uint32_t ub_cand;
   uint32_t s2_done;
+  uint32_t ptasks;  // pieces of rows in which parents are still looked for
   uint32_t next_q;  // batch: the query the group's first block claimed
   unsigned long long next_ticket;  // serving: the request the group's first block claimed
   uint32_t acc_maxd1;  // 1 + the largest distance settled in the step (0: none)

@@ -2117,6 +2117,7 @@ __device__ void ctl_init(const KArgs& A, bool set_source) {
   c->touched_cnt = 1;
   c->ub_cand = (G.highd0 > 0 && dgs >= G.highd0) ? 0u : EIC_INF;
   c->s2_done = 0;
+  c->ptasks = 0;
   c->acc_maxd1 = 0;
   c->acc_deg = 0;
   c->cnt_rounds = c->cnt_frontier = c->cnt_trav = c->cnt_pulls = c->cnt_improved = c->cnt_heavy = 0;
@@ -2172,38 +2173,85 @@ __global__ void k_output(DevGraph G, const uint32_t* __restrict__ idist, uint32_
 }
 
 // parent[v] = smallest original id u with dist[u] + w(u, v) == dist[v]; parent[s]
-// = s, +inf where unreachable. Bound by the chain id -> distance -> entries ->
-// their distances of every vertex, and by the longest row: eight lanes take a
-// row (a warp's 32 mostly idled), and rows of more than kBigRow entries, which
-// come first in the adjacency, are shared out over the grid by k_parent_big.
-// With parents a query of an RMAT graph of 250 k vertices (longest row 24 k)
-// takes 52 us longer (159 before), of 2^22 402 us (652), of 2^25 4.4 ms (9.1).
+// = s, +inf where unreachable. Only the prefix of v's row with weight <= dist[v]
+// can hold u. Bound by the chain id -> distance -> entries -> their distances of
+// every vertex, and by the longest prefix: eight lanes take a row (a warp's 32
+// mostly idled); a row of more than kBigRow entries (these come first) is taken
+// by a warp, 128 entries at a time, and what its prefix holds beyond kParentAlone
+// is shared out over the grid in pieces. With parents a query of a dense graph
+// (32 k vertices, 256 M entries) takes 22 us longer, of RMAT graphs of 250 k
+// vertices 29, of 2^22 236, of 2^25 1.60 ms; 592, 37, 395 us and 3.19 ms when
+// every entry of the big rows was read, 23, 43, 582 us and 6.28 ms when a warp
+// took every row. kBigRow 128, 256 and 512: rows of 500 entries (5 k vertices,
+// unit weights) 18, 18 and 45 us, rows of 128 (512 k vertices) 137, 94 and 92.
 constexpr uint32_t kParentLanes = 8;
-constexpr uint32_t kBigChunk = 256;  // entries of the big rows a warp takes at a time
+constexpr uint32_t kParentAlone = 512;
+constexpr uint32_t kParentPiece = 256;
+static_assert(kParentAlone >= kParentPiece && kParentPiece >= kHeavyMinFloor,
+              "a row has at most length / kParentPiece pieces, and the task list 2m / kHeavyMinFloor entries");
 
-// best[vi] (all ones before): the parent of the vertices with big rows.
-__global__ void k_parent_big(DevGraph G, const uint32_t* __restrict__ idist, uint32_t* best) {
-  const uint32_t lane = lane_id(), wpb = blockDim.x >> 5;
-  const uint64_t nw = (uint64_t)gridDim.x * wpb;
-  for (uint64_t at = ((uint64_t)blockIdx.x * wpb + (threadIdx.x >> 5)) * kBigChunk; at < G.big_end; at += nw * kBigChunk) {
-    uint32_t lo = 0, hi = G.nbig - 1;  // the row that holds the chunk's first entry
-    while (lo < hi) {
-      const uint32_t mid = (lo + hi + 1) >> 1;
-      if (__ldg(&G.row[mid]) <= at)
-        lo = mid;
-      else
-        hi = mid - 1;
+// The smallest parent among kIlp entries per lane of the row part [at, at + len); last: the weight of the last entry
+// looked at (all ones past the part's end).
+template <uint32_t kIlp>
+__device__ __forceinline__ uint32_t parent_of(const DevGraph& G, const uint32_t* __restrict__ idist, uint32_t at,
+                                              uint32_t len, uint32_t dv, uint32_t* last) {
+  const uint32_t lane = lane_id();
+  uint2 ent[kIlp];
+  uint32_t du[kIlp], best = EIC_INF;
+#pragma unroll
+  for (uint32_t j = 0; j < kIlp; ++j)
+    ent[j] = 32 * j + lane < len ? ld_stream(&G.adj[at + 32 * j + lane]) : make_uint2(0u, EIC_INF);
+#pragma unroll
+  for (uint32_t j = 0; j < kIlp; ++j) du[j] = ent[j].y <= dv ? __ldg(&idist[ent[j].x]) : EIC_INF;
+#pragma unroll
+  for (uint32_t j = 0; j < kIlp; ++j)
+    if (du[j] != EIC_INF && (uint64_t)du[j] + ent[j].y == dv) best = min(best, __ldg(&G.int2orig[ent[j].x]));
+  *last = __shfl_sync(EIC_FULL_MASK, ent[kIlp - 1].y, 31);
+  return best;
+}
+
+// best[vi] for the vertices with big rows, from the first kParentAlone entries; the rest of their prefixes to tasks.
+__global__ void __launch_bounds__(256) k_parent_big(DevGraph G, const uint32_t* __restrict__ idist, uint32_t* best,
+                                                    Task* tasks, uint32_t* count) {
+  const uint32_t lane = lane_id(), nw = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t vi = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); vi < G.nbig; vi += nw) {
+    const uint32_t dv = __ldg(&idist[vi]), end = __ldg(&G.row[vi + 1]);
+    uint32_t at = __ldg(&G.row[vi]), mine = EIC_INF, last = 0;
+    bool more = dv != EIC_INF;  // the prefix goes on at `at`
+    for (uint32_t k = 0; more && k < kParentAlone; k += 128) {
+      mine = min(mine, parent_of<4>(G, idist, at, end - at, dv, &last));
+      more = last <= dv;  // (then all 128 entries were there)
+      at += more ? 128u : 0u;
     }
-    const uint64_t end = min(at + kBigChunk, (uint64_t)G.big_end);
-    uint32_t vi = lo, re = __ldg(&G.row[lo + 1]);
-    for (uint64_t i = at + lane; i < end; i += 32) {
-      while (i >= re) re = __ldg(&G.row[++vi + 1]);
-      const uint32_t dv = __ldg(&idist[vi]);
-      const uint2 ent = __ldg(&G.adj[i]);
-      if (dv == EIC_INF || ent.y > dv) continue;
-      const uint32_t du = __ldg(&idist[ent.x]);
-      if (du != EIC_INF && (uint64_t)du + ent.y == dv) atomicMin(&best[vi], __ldg(&G.int2orig[ent.x]));
+    mine = __reduce_min_sync(EIC_FULL_MASK, mine);
+    if (lane == 0) best[vi] = mine;
+    if (!more) continue;
+    uint32_t lo = at, hi = end;  // the prefix's end, by 32 probes at a time
+    while (hi - lo > 32) {
+      const uint32_t step = (hi - lo + 32) / 33, off = (lane + 1) * step;
+      const uint32_t in = __popc(__ballot_sync(EIC_FULL_MASK, off < hi - lo && ld_stream_w(&G.adj[lo + off]) <= dv));
+      hi = in < 32 && (in + 1) * step < hi - lo ? lo + (in + 1) * step : hi;
+      lo += in ? in * step + 1 : 0u;
     }
+    lo += __popc(__ballot_sync(EIC_FULL_MASK, lane < hi - lo && ld_stream_w(&G.adj[lo + lane]) <= dv));
+    const uint32_t len = lo - at, nt = (len + kParentPiece - 1) / kParentPiece;
+    uint32_t slot = 0;
+    if (lane == 0 && nt) slot = atomicAdd(count, nt);
+    slot = __shfl_sync(EIC_FULL_MASK, slot, 0);
+    for (uint32_t k = lane; k < nt; k += 32)
+      tasks[slot + k] = Task{at + k * kParentPiece, min(kParentPiece, len - k * kParentPiece), vi, dv};
+  }
+}
+
+__global__ void __launch_bounds__(256) k_parent_pieces(DevGraph G, const uint32_t* __restrict__ idist,
+                                                       const Task* __restrict__ tasks,
+                                                       const uint32_t* __restrict__ count, uint32_t* best) {
+  const uint32_t nw = gridDim.x * (blockDim.x >> 5), n = __ldg(count);
+  for (uint32_t k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < n; k += nw) {
+    const uint4 t = __ldg(reinterpret_cast<const uint4*>(&tasks[k]));
+    uint32_t last;
+    const uint32_t mine = __reduce_min_sync(EIC_FULL_MASK, parent_of<kParentPiece / 32>(G, idist, t.x, t.y, t.w, &last));
+    if (lane_id() == 0 && mine != EIC_INF) atomicMin(&best[t.z], mine);
   }
 }
 
@@ -2720,10 +2768,11 @@ int enqueue_query(eic_graph* g, uint32_t s, uint32_t* dist, uint32_t* parent, co
   k_output<<<4 * w.grid, 256, 0, st>>>(g->dg, w.idist, s, dist);
   EIC_CUDA_TRY(cudaGetLastError());
   if (parent) {
-    if (g->dg.nbig) {  // (the queue's words have served)
-      EIC_CUDA_TRY(cudaMemsetAsync(w.q[0], 0xFF, (uint64_t)g->dg.nbig * 4, st));
-      k_parent_big<<<(unsigned)std::min<uint64_t>(8 * w.sms, g->dg.big_end / (8 * kBigChunk) + 1), 256, 0, st>>>(
-          g->dg, w.idist, w.q[0]);
+    if (g->dg.nbig) {  // (the queue's words and the tasks have served)
+      k_parent_big<<<std::min(8 * (unsigned)w.sms, g->dg.nbig / 8 + 1), 256, 0, st>>>(g->dg, w.idist, w.q[0], w.tasks,
+                                                                                     &w.ctl->ptasks);
+      k_parent_pieces<<<std::min(8 * (unsigned)w.sms, g->dg.big_end / (8 * kParentPiece) + 1), 256, 0, st>>>(
+          g->dg, w.idist, w.tasks, &w.ctl->ptasks, w.q[0]);
     }
     k_parent<<<(unsigned)std::min<uint64_t>(8 * w.sms, (uint64_t)g->dg.n / 32 + 1), 256, 0, st>>>(g->dg, w.idist, w.q[0],
                                                                                                   s, parent);
