@@ -2269,8 +2269,8 @@ __global__ void k_parent(DevGraph G, const uint32_t* __restrict__ idist, const u
       } else {
         const uint32_t dv = __ldg(&idist[vi]);
         const uint2 rr = dv != EIC_INF ? row_of(G, vi) : make_uint2(0u, 0u);
-        for (uint32_t i = rr.x + sub; i < rr.x + rr.y; i += kParentLanes) {
-          const uint2 ent = __ldg(&G.adj[i]);
+        for (uint32_t k = sub; k < rr.y; k += kParentLanes) {  // (an entry's index plus the step may wrap)
+          const uint2 ent = __ldg(&G.adj[rr.x + k]);
           if (ent.y > dv) break;  // (rows are in weight order)
           const uint32_t du = __ldg(&idist[ent.x]);
           if (du != EIC_INF && (uint64_t)du + ent.y == dv) best = min(best, __ldg(&G.int2orig[ent.x]));
