@@ -2669,10 +2669,16 @@ struct DeviceGuard {
 // isolated) 698, 672; 2 M 806, 804; 4 M 957, 1034; uniform 16 k 399, 368; 131 k
 // 506, 509; 1 M 813, 841; grids 1024^2 24.1, 23.1 ms; 2048^2 46.9, 44.6; at
 // gap_shift 4 1000^2 4.95, 4.80, 3000^2 15.6, 15.8.
+// A dense graph with few distinct weights is no chain of small steps however
+// few its vertices: the rows' entries of one weight, about 2m / maxW, all fall
+// into the same step. 8 k to 260 k vertices with 41, 46, 50, 83, 132 and 208 M
+// entries of weight 1: 560, 509, 485, 593, 801, 1114 us with 304 blocks and 467,
+// 504, 604, 805, 1139, 1714 with 152; 266 M of weights up to 4: 641, 915; up to
+// 8 (33 M each): 299, 317; up to 255: 302, 294.
 int query_blocks(const DevGraph& G, const eic_params& p, int block, int sms, int per_sm) {
   const uint64_t vertices = (uint64_t)G.ni << p.gap_shift;  // (wider steps settle more at a time)
-  const uint64_t most = fuse_items(G, p.heavy_min, p.flags) == kFuseRoad ? 1ull << 26 : 3ull << 18;
-  if (vertices > most) return sms * per_sm;
+  const bool road = fuse_items(G, p.heavy_min, p.flags) == kFuseRoad;
+  if (vertices > (road ? 1ull << 26 : 3ull << 18) || (!road && G.two_m / G.maxw > 45u << 20)) return sms * per_sm;
   return sms * std::min(per_sm, std::max(1, kDefaultBlock / block));
 }
 
