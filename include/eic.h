@@ -53,8 +53,8 @@ typedef struct eic_graph eic_graph;
  *   heavy_min     window length above which a vertex's edges are cut into
  *                 64-entry tasks spread over the whole grid instead of being
  *                 relaxed by one warp (0 = library choice, 32; else 16..4096).
- *   max_spin_log2 bound on each grid-barrier wait, 2^max_spin_log2 polls of
- *                 about 100 ns (0 = library choice, about 2 s); exceeding it
+ *   max_spin_log2 bound on each grid-barrier wait, 2^max_spin_log2 times about
+ *                 0.5 us (0 = library choice, 22: about 2 s); exceeding it
  *                 returns EIC_ETIMEOUT.
  *   flags         EIC_FLAG_* bits.
  *   batch_groups  batches only: number of block groups that run queries at

@@ -184,7 +184,7 @@ struct eic_server {
     a.flags = p.flags;
     a.step_cap = kServeStepCap;
     const uint32_t sl = p.max_spin_log2 > kServeSpinLog2 ? p.max_spin_log2 : kServeSpinLog2;
-    a.max_spin = 1ull << sl;
+    a.max_spin = spin_limit(sl);
     a.groups = g;
     a.wide = wide;
     a.idle_ns = idle_ns;

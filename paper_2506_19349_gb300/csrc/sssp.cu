@@ -2736,7 +2736,7 @@ KArgs make_args(eic_graph* g, uint32_t s, uint32_t* dist, const eic_params& p, i
   A.st_num = p.st_num;
   A.gap_shift = p.gap_shift;
   A.heavy_min = p.heavy_min;
-  A.max_spin = 1ull << p.max_spin_log2;
+  A.max_spin = spin_limit(p.max_spin_log2);
   A.flags = p.flags;
   A.ring_mask = (1u << w.ring_bits) - 1u;
   A.ring_shift = w.ring_shift;
@@ -3103,7 +3103,7 @@ BatchArgs batch_args(const eic_batch* b) {
   P.heavy_min = b->p.heavy_min;
   P.flags = b->p.flags;
   P.step_cap = kBatchStepCap;
-  P.max_spin = 1ull << b->p.max_spin_log2;
+  P.max_spin = spin_limit(b->p.max_spin_log2);
   return P;
 }
 
@@ -3616,7 +3616,7 @@ extern "C" int eic_sssp_noalloc(const eic_graph* gc, uint32_t source, uint32_t* 
   A.st_num = 1024;
   A.gap_shift = 0;
   A.heavy_min = kDefaultHeavyMin;
-  A.max_spin = 1ull << kDefaultSpinLog2;
+  A.max_spin = spin_limit(kDefaultSpinLog2);
   A.flags = 0;
   A.ring_mask = (1u << kNaRingBits) - 1u;
   A.ring_shift = 0;
