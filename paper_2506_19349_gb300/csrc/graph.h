@@ -124,6 +124,8 @@ struct Workspace {
   unsigned long long* timeline = nullptr;
   Ctl* ctl = nullptr;
   Ctl* ctl_host = nullptr;  // pinned mirror for status readback
+  struct PinnedSlots* ctl_pool = nullptr;  // ... a slot of this pool's epoch, or (nullptr) an allocation of its own
+  uint64_t ctl_epoch = 0;
   cudaEvent_t ev[2] = {nullptr, nullptr};  // around the query kernel, when statistics are asked for
   uint32_t ring_bits = 0, ring_shift = 0;
   uint32_t task_cap = 0, step_cap = 0;

@@ -2,6 +2,8 @@
 // of one group's arrays, and a pool of groups in one device allocation.
 #pragma once
 
+#include <string.h>
+
 #include <mutex>
 #include <vector>
 
@@ -9,6 +11,7 @@
 
 constexpr uint32_t kBatchStepCap = 1u << 17;  // steps per query of a batch
 constexpr double kBatchMemFrac = 0.8;         // share of free device memory the scratch may take
+constexpr int kMaxDevices = 64;
 
 // Capacities one block group's scratch must cover.
 struct SlotCaps {
@@ -117,35 +120,65 @@ struct SlotPool {
   }
 };
 
-// Pinned host mirrors of control blocks: 128 slots of one small allocation,
-// made at the first use and kept, since page-locking and unlocking a few
-// hundred bytes takes 0.3 ms a graph. get() gives nullptr when every slot is
-// taken; put() takes back a slot of this pool and says whether it was one.
+// Pinned host mirrors of a device's control blocks: 127 slots of one small
+// allocation, made at the first use and kept, since page-locking and unlocking
+// a few hundred bytes takes 0.3 ms a graph. get() gives nullptr when every slot
+// is taken; put() takes a slot back. The allocation goes with the device's
+// context (cudaDeviceReset): get() then makes a new one, which it tells from
+// the old by its epoch, and slots of an earlier epoch are forgotten.
 struct PinnedSlots {
-  static constexpr uint32_t kSlots = 128, kBytes = 512;
+  static constexpr uint32_t kSlots = 128, kBytes = 512;  // (slot 0 holds the mark)
   std::mutex mu;
   unsigned char* base = nullptr;
+  uint64_t epoch = 0;
   uint64_t taken[kSlots / 64] = {};
-  void* get() {
-    std::lock_guard<std::mutex> lock(mu);
-    if (!base && cudaHostAlloc((void**)&base, kSlots * kBytes, cudaHostAllocPortable) != cudaSuccess) {
+
+  struct Mark {
+    const void* pool;
+    uint64_t epoch, check;
+  };
+  Mark mark() const { return {this, epoch, 0x6569635f736c6f74ull ^ epoch}; }
+
+  // The allocation is still page-locked memory, and this pool's.
+  bool alive() const {
+    cudaPointerAttributes a;
+    if (!base || cudaPointerGetAttributes(&a, base) != cudaSuccess || a.type != cudaMemoryTypeHost) {
       (void)cudaGetLastError();
+      return false;
+    }
+    const Mark want = mark();
+    return memcmp(base, &want, sizeof(Mark)) == 0;
+  }
+
+  void* get(uint64_t* slot_epoch) {
+    std::lock_guard<std::mutex> lock(mu);
+    if (!alive()) {
       base = nullptr;
-      return nullptr;
+      if (cudaHostAlloc((void**)&base, kSlots * kBytes, cudaHostAllocPortable) != cudaSuccess) {
+        (void)cudaGetLastError();
+        base = nullptr;
+        return nullptr;
+      }
+      ++epoch;
+      const Mark m = mark();
+      memcpy(base, &m, sizeof(Mark));
+      memset(taken, 0, sizeof(taken));
+      taken[0] = 1;
     }
     for (uint32_t k = 0; k < kSlots; ++k)
       if (!(taken[k / 64] >> (k % 64) & 1)) {
         taken[k / 64] |= 1ull << (k % 64);
+        *slot_epoch = epoch;
         return base + k * kBytes;
       }
     return nullptr;
   }
-  bool put(void* p) {
+
+  void put(void* p, uint64_t slot_epoch) {
     std::lock_guard<std::mutex> lock(mu);
-    const uint64_t off = (uint64_t)((unsigned char*)p - base);
-    if (!base || (unsigned char*)p < base || off >= kSlots * kBytes) return false;
-    taken[off / kBytes / 64] &= ~(1ull << (off / kBytes % 64));
-    return true;
+    if (slot_epoch != epoch || !base) return;
+    const uint64_t k = (uint64_t)((unsigned char*)p - base) / kBytes;
+    taken[k / 64] &= ~(1ull << (k % 64));
   }
 };
 

@@ -2831,12 +2831,15 @@ int output_view(int dev, uint32_t* p, uint32_t** out) {
 }  // namespace
 
 namespace {
-PinnedSlots g_mirrors;
+PinnedSlots g_mirrors[kMaxDevices];
 }  // namespace
 
 void eic_ws_free(Workspace* w) {
   cudaFree(w->base);
-  if (w->ctl_host && !g_mirrors.put(w->ctl_host)) cudaFreeHost(w->ctl_host);
+  if (w->ctl_pool)
+    w->ctl_pool->put(w->ctl_host, w->ctl_epoch);
+  else if (w->ctl_host)
+    cudaFreeHost(w->ctl_host);
   if (w->ev[0]) cudaEventDestroy(w->ev[0]);
   if (w->ev[1]) cudaEventDestroy(w->ev[1]);
   *w = Workspace();
@@ -2886,7 +2889,9 @@ int eic_ws_ensure(eic_graph* g, int) {
   w->trace = (eic_step*)(b + trace);
   w->timeline = (unsigned long long*)(b + timeline);
   static_assert(sizeof(Ctl) <= PinnedSlots::kBytes, "a control block fits a slot");
-  w->ctl_host = (Ctl*)g_mirrors.get();
+  PinnedSlots* pool = g->device >= 0 && g->device < kMaxDevices ? &g_mirrors[g->device] : nullptr;
+  w->ctl_host = pool ? (Ctl*)pool->get(&w->ctl_epoch) : nullptr;
+  w->ctl_pool = w->ctl_host ? pool : nullptr;
   if (!w->ctl_host && cudaMallocHost((void**)&w->ctl_host, sizeof(Ctl)) != cudaSuccess) {
     (void)cudaGetLastError();
     eic_ws_free(w);
@@ -2894,10 +2899,6 @@ int eic_ws_ensure(eic_graph* g, int) {
   }
   return EIC_OK;
 }
-
-namespace {
-constexpr int kMaxDevices = 64;
-}  // namespace
 
 extern "C" {
 
