@@ -92,11 +92,13 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_radix_scatter(const uint64_
                                                                    uint32_t* __restrict__ vals_out) {
   __shared__ uint64_t s_k[kSortTile];
   __shared__ uint32_t s_v[kHasVals ? kSortTile : 1];
-  __shared__ uint16_t s_c[kSortWarps][kRadixDigits];  // per warp and digit: the tile's elements, then those of earlier warps
+  // per warp and digit: the tile's elements, then those of earlier warps (cleared two digits at a time)
+  __shared__ __align__(4) uint16_t s_c[kSortWarps][kRadixDigits];
   __shared__ uint32_t s_start[kRadixDigits];          // a digit's first place in the tile
   __shared__ uint32_t s_out[kRadixDigits];            // ... and in the output, minus s_start
   __shared__ uint32_t s_w[32];
   static_assert(kRadixDigits <= kSortThreads, "one thread per digit");
+  static_assert(kRadixDigits % 2 == 0, "a warp's row of s_c starts on a word");
   const uint32_t t = threadIdx.x, w = t >> 5, lane = t & 31u, lt = (1u << lane) - 1u;
   uint32_t sum;
   // the output place of the slice's next element of digit t
