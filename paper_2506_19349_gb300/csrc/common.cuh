@@ -35,7 +35,6 @@ struct DevGraph {
   uint64_t m;             // undirected edges
   const uint32_t* row;    // [ni + 1] row offsets (2m < 2^32)
   const uint2* adj;       // [two_m] {neighbour, weight}, rows sorted by (weight, neighbour)
-  const uint32_t* drank;  // [max_deg + 1] degree -> rank among distinct degrees (present ones)
   const uint32_t* dvals;  // [D] distinct degrees >= 1, ascending
   const uint32_t* dcnt0;  // [D] number of vertices with degree dvals[r]
   const uint32_t* dfirst;  // [D] first internal id of degree dvals[r] (decreasing in r: ids run by degree descending)

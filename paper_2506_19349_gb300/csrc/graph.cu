@@ -372,16 +372,12 @@ __global__ void k_flag_present(const uint32_t* __restrict__ hist, uint32_t len, 
 }
 
 __global__ void k_degree_tables(const uint32_t* __restrict__ hist, const uint32_t* __restrict__ flags,
-                                const uint64_t* __restrict__ pos, uint32_t len, uint32_t* dvals, uint32_t* dcnt0,
-                                uint32_t* drank) {
+                                const uint64_t* __restrict__ pos, uint32_t len, uint32_t* dvals, uint32_t* dcnt0) {
   for (uint32_t d = blockIdx.x * blockDim.x + threadIdx.x; d < len; d += gridDim.x * blockDim.x) {
     if (flags[d]) {
-      uint32_t r = (uint32_t)pos[d];
+      const uint32_t r = (uint32_t)pos[d];
       dvals[r] = d;
       dcnt0[r] = hist[d];
-      drank[d] = r;
-    } else {
-      drank[d] = 0xFFFFFFFFu;
     }
   }
 }
@@ -477,7 +473,6 @@ int galloc(eic_graph* g, T** out, uint64_t count) {
 void graph_free_arrays(eic_graph* g) {
   cudaFree(g->row);
   cudaFree(g->adj);
-  cudaFree(g->drank);
   cudaFree(g->dvals);
   cudaFree(g->dcnt0);
   cudaFree(g->dfirst);
@@ -673,8 +668,7 @@ int build(eic_graph* g, const uint32_t* src, const uint32_t* dst, const uint32_t
     D = (uint32_t)dd;
     TRY(galloc(g, &g->dvals, D));
     TRY(galloc(g, &g->dcnt0, D));
-    TRY(galloc(g, &g->drank, hlen));
-    k_degree_tables<<<grid_for(hlen), kThreads, 0, st>>>(dh, flags, pos, hlen, g->dvals, g->dcnt0, g->drank);
+    k_degree_tables<<<grid_for(hlen), kThreads, 0, st>>>(dh, flags, pos, hlen, g->dvals, g->dcnt0);
     k_highd0<<<1, 1024, 0, st>>>(g->dcnt0, g->dvals, D, small + 5);
     EIC_CUDA_TRY(cudaGetLastError());
     // dfirst[r]: the first internal id of degree dvals[r] (ids by degree descending); drow[r]: the same with that
@@ -768,7 +762,6 @@ int build(eic_graph* g, const uint32_t* src, const uint32_t* dst, const uint32_t
   dg.m = m;
   dg.row = g->row;
   dg.adj = g->adj;
-  dg.drank = g->drank;
   dg.dvals = g->dvals;
   dg.dcnt0 = g->dcnt0;
   dg.dfirst = g->dfirst;

@@ -6,7 +6,8 @@
 #include "common.cuh"
 
 // Smallest accepted heavy_min: a window longer than it yields at most len / 16
-// tasks, which bounds every task list at 2m / 16 entries.
+// tasks, and the windows of one round belong to distinct vertices, which bounds
+// every task list at 2m / 16 entries.
 constexpr uint32_t kHeavyMinFloor = 16;
 
 // A window of at most kTaskLen adjacency entries relaxed by one warp in a
@@ -39,10 +40,7 @@ struct Ctl {
   uint32_t pull_sweep;  // the pull set is swept in vertex order (pull_cnt = all vertices; the round takes the unsettled ones)
   uint32_t step_off_cur;  // settled-list offset where the current step's vertices start
   // private to the step-boundary block
-  int64_t st0, st1, gap_lb;
-  uint64_t sumd_lb, highd_lb;
-  int64_t max_settled;
-  uint32_t rounds_in_step;
+  int64_t gap_lb;  // of the first step
   uint32_t trace_len;
   uint32_t tl_len;  // diagnostic timeline events recorded
   // appended with atomics during phases
@@ -67,7 +65,7 @@ struct BatchQuery {
   DevGraph G;
   uint32_t* out;
   uint32_t s;
-  uint32_t ring_mask, ring_shift, task_cap;
+  uint32_t ring_mask, ring_shift;
   uint32_t gap_shift, heavy_min;  // step-width scaling and window-class threshold for this query's graph
   uint32_t fuse;                  // rounds of at most this many items per warp are fused (fuse_items)
 };
@@ -128,7 +126,7 @@ struct Workspace {
   uint64_t ctl_epoch = 0;
   cudaEvent_t ev[2] = {nullptr, nullptr};  // around the query kernel, when statistics are asked for
   uint32_t ring_bits = 0, ring_shift = 0;
-  uint32_t task_cap = 0, step_cap = 0;
+  uint32_t step_cap = 0;
   uint64_t bytes = 0;
   int grid = 0, block = 0, sms = 0;  // co-resident blocks of k_eic at this block size, and the SMs
 };
@@ -138,7 +136,6 @@ struct eic_graph {
   DevGraph dg{};
   uint32_t* row = nullptr;
   uint2* adj = nullptr;
-  uint32_t* drank = nullptr;
   uint32_t* dvals = nullptr;
   uint32_t* dcnt0 = nullptr;
   uint32_t* dfirst = nullptr;

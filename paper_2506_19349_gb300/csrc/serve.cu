@@ -387,7 +387,6 @@ int eic_server_create(const eic_graph* const* graphs, uint32_t num_graphs, const
     s->wide |= shift != 0;
     q.ring_mask = (1u << bits) - 1u;
     q.ring_shift = shift;
-    q.task_cap = (uint32_t)(G.two_m / kHeavyMinFloor + 2);
     q.gap_shift = pr.gap_shift;
     q.heavy_min = pr.heavy_min;
     q.fuse = fuse_items(G, pr.heavy_min, pr.flags);

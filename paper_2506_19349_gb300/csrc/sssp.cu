@@ -91,7 +91,7 @@ struct KArgs {
   uint64_t max_spin;
   uint32_t flags;
   uint32_t ring_mask, ring_shift;
-  uint32_t task_cap, step_cap, trace_cap;
+  uint32_t step_cap, trace_cap;
   unsigned long long* timeline;  // NULL unless the caller asked for it
   uint32_t timeline_cap;
   uint32_t nb;  // blocks working on this query: the grid, or one block group of a batch
@@ -439,20 +439,17 @@ __device__ __forceinline__ void emit_tasks_warp(const KArgs& A, const RoundCtx& 
   }
 }
 
-// Successful relaxation of v to nd (old = previous distance): SAP into the
-// next frontier, first insertion into the settled (or first-step) list, and
-// in the first step the running min over high-degree vertices that becomes
-// ub (Algorithm 1). Warp-collective: every lane calls it; the appends go
-// through the warp's stages.
 // Sets v's bit in the round's insertion bitmap; true when this call set it.
 __device__ __forceinline__ bool claim_bit(const RoundCtx& R, uint32_t v) {
   const uint32_t bit = 1u << (v & 31);
   return !(atomicOr(&R.fbits[v >> 5], bit) & bit);
 }
 
-// After a relaxation: v into the next frontier when sap (its insertion bit was
-// set by this lane), into the first-reached list when it had no distance, and
-// the first step's ub candidate when v's degree is at least highD(0).
+// After a relaxation of v to nd (old = its previous distance): v into the next
+// frontier when sap (its insertion bit was set by this lane), into the settled
+// (or first-step) list when it had no distance, and in the first step the
+// running min over high-degree vertices that becomes ub (Algorithm 1).
+// Warp-collective: every lane calls it; the appends go through the warp's stages.
 __device__ __forceinline__ void on_claimed(const KArgs& A, const RoundCtx& R, bool ok, bool sap, uint32_t v,
                                            uint32_t nd, uint32_t old, Counters& C, WarpList& Q, WarpList& F) {
   const bool first = ok && old == EIC_INF;
@@ -465,21 +462,11 @@ __device__ __forceinline__ void on_claimed(const KArgs& A, const RoundCtx& R, bo
   C.improved += ok ? 1 : 0;
 }
 
+// The same for a relaxation (ok: it lowered v's distance) whose bit is not yet claimed.
 __device__ __forceinline__ void on_success(const KArgs& A, const RoundCtx& R, bool ok, uint32_t v, uint32_t nd,
                                            uint32_t old, Counters& C, WarpList& Q, WarpList& F) {
-  bool sap = false;
-  if (ok) {
-    const uint32_t bit = 1u << (v & 31);
-    sap = !(atomicOr(&R.fbits[v >> 5], bit) & bit);
-  }
-  const bool first = ok && old == EIC_INF;
-  warp_push(Q, sap, v);
-  warp_push(F, first, v);
-  if (R.step1 && ok) {
-    const uint32_t dg = __ldg(&A.G.row[v + 1]) - __ldg(&A.G.row[v]);
-    if (dg >= A.G.highd0) atomicMin(&A.ctl->ub_cand, nd);
-  }
-  C.improved += ok ? 1 : 0;
+  const bool sap = ok && claim_bit(R, v);
+  on_claimed(A, R, ok, sap, v, nd, old, C, Q, F);
 }
 
 // One round over nitems items. Items are frontier vertices (queue qin), or in
@@ -1079,8 +1066,8 @@ __device__ __noinline__ int64_t block_st_bins(uint32_t* bins, uint32_t st_num, u
 // round: uniform 2^14 vertices 488 -> 394 us, RMAT 131 k 579 -> 518 us, RMAT
 // 2^22 1029 -> 990 us, RMAT 2^25 3.03 -> 2.94 ms a query.
 template <bool kRoad>
-__device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, RoundScr& S, Stage& T,
-                            uint32_t nitems, bool round1, const uint32_t* qin, Counters& C) {
+__device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, Stage& T, uint32_t nitems, bool round1,
+                            const uint32_t* qin, Counters& C) {
   const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
   const uint32_t wpb = blockDim.x >> 5, gpb = (wpb + kFuseWarps - 1) / kFuseWarps;
   const uint32_t grp = warp / kFuseWarps, gw = warp - grp * kFuseWarps;  // the group, the warp's place in it
@@ -1854,9 +1841,9 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ti
       if (qb == 0 && threadIdx.x == 0) tl_mark(A, 8, nitems);  // diagnostic: the round's items
       if (!R.step1 && (!round1 || !LL.pull_on) && !plain && nitems <= A.fuse * A.nb * (blockDim.x >> 5)) {
         if (A.fuse == kFuseRoad)
-          fused_round<true>(A, R, LL, P.r, T, nitems, round1, qin, C);
+          fused_round<true>(A, R, LL, T, nitems, round1, qin, C);
         else
-          fused_round<false>(A, R, LL, P.r, T, nitems, round1, qin, C);
+          fused_round<false>(A, R, LL, T, nitems, round1, qin, C);
       } else {
         round_phase<kPullFast, kRelaxIlp>(A, R, LL, P.r, T, nitems, round1, qin, C);
       }
@@ -2103,13 +2090,7 @@ __device__ void ctl_init(const KArgs& A, bool set_source) {
   c->pull_on = c->pull_cnt = c->extra_s = 0;
   c->pull_sweep = 0;
   c->step_off_cur = 0;
-  c->st0 = -1;
-  c->st1 = -1;
-  c->sumd_lb = G.two_m;
-  c->highd_lb = G.highd0;
   c->gap_lb = dev_gap(G.two_m, G.highd0, G.two_m, A.alpha, A.beta, G.rtow);
-  c->max_settled = -1;
-  c->rounds_in_step = 0;
   c->trace_len = 0;
   c->tl_len = 0;
   c->rcnt[0] = c->rcnt[1] = c->rcnt[2] = make_uint4(0u, 0u, 0u, 0u);
@@ -2377,7 +2358,6 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_batch(BatchArgs P) {
       sA.flags = P.flags;
       sA.ring_mask = bq.ring_mask;
       sA.ring_shift = bq.ring_shift;
-      sA.task_cap = bq.task_cap;
       sA.step_cap = P.step_cap;
       sA.trace_cap = 0;
       sA.timeline = nullptr;
@@ -2564,7 +2544,6 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_eic_serve(ServeArgs P) {
       sA.flags = P.flags;
       sA.ring_mask = bq.ring_mask;
       sA.ring_shift = bq.ring_shift;
-      sA.task_cap = bq.task_cap;
       sA.step_cap = P.step_cap;
       sA.trace_cap = 0;
       sA.timeline = nullptr;
@@ -2740,7 +2719,6 @@ KArgs make_args(eic_graph* g, uint32_t s, uint32_t* dist, const eic_params& p, i
   A.flags = p.flags;
   A.ring_mask = (1u << w.ring_bits) - 1u;
   A.ring_shift = w.ring_shift;
-  A.task_cap = w.task_cap;
   A.step_cap = w.step_cap;
   A.trace_cap = kTraceCap;
   A.timeline = nullptr;
@@ -2850,9 +2828,6 @@ int eic_ws_ensure(eic_graph* g, int) {
   if (w->ctl) return EIC_OK;
   const DevGraph& G = g->dg;
   w->ring_bits = ring_layout(G.maxw, &w->ring_shift);
-  // a window longer than heavy_min >= 16 yields ceil(len / 64) <= len / 16 tasks,
-  // and the windows of one round belong to distinct vertices
-  w->task_cap = (uint32_t)(G.two_m / kHeavyMinFloor + 2);
   w->step_cap = kStepCap;
   w->n = G.ni;  // per-vertex arrays cover the internal (non-isolated) vertices
   SlotCaps caps;
@@ -3178,7 +3153,6 @@ int batch_create(const eic_graph* const* graphs, const uint32_t* sources, uint32
     b->wide |= shift != 0;
     q.ring_mask = (1u << bits) - 1u;
     q.ring_shift = shift;
-    q.task_cap = (uint32_t)(G.two_m / kHeavyMinFloor + 2);
     q.gap_shift = p.gap_shift;
     q.heavy_min = p.heavy_min;
     q.fuse = fuse_items(G, p.heavy_min, p.flags);
@@ -3621,7 +3595,6 @@ extern "C" int eic_sssp_noalloc(const eic_graph* gc, uint32_t source, uint32_t* 
   A.flags = 0;
   A.ring_mask = (1u << kNaRingBits) - 1u;
   A.ring_shift = 0;
-  A.task_cap = (uint32_t)kNaTasks;
   A.step_cap = (uint32_t)kNaS;
   A.trace_cap = 0;
   A.timeline = nullptr;
