@@ -2653,10 +2653,12 @@ struct DeviceGuard {
 // into the same step. 8 k to 260 k vertices with 41, 46, 50, 83, 132 and 208 M
 // entries of weight 1: 560, 509, 485, 593, 801, 1114 us with 304 blocks and 467,
 // 504, 604, 805, 1139, 1714 with 152; 266 M of weights up to 4: 641, 915; up to
-// 8 (33 M each): 299, 317; up to 255: 302, 294.
+// 8 (33 M each): 299, 317; up to 255: 302, 294. Nor is a graph of small degrees
+// whose average is above 8 (no road network's is): 1 M vertices of degree 30
+// without pulls 694, 744; 2 M 1019, 1047; 4 M of degree 16 1489, 1600.
 int query_blocks(const DevGraph& G, const eic_params& p, int block, int sms, int per_sm) {
   const uint64_t vertices = (uint64_t)G.ni << p.gap_shift;  // (wider steps settle more at a time)
-  const bool road = fuse_items(G, p.heavy_min, p.flags) == kFuseRoad;
+  const bool road = fuse_items(G, p.heavy_min, p.flags) == kFuseRoad && G.two_m <= 8ull * G.ni;
   if (vertices > (road ? 1ull << 26 : 3ull << 18) || (!road && G.two_m / G.maxw > 45u << 20)) return sms * per_sm;
   return sms * std::min(per_sm, std::max(1, kDefaultBlock / block));
 }
