@@ -1193,7 +1193,7 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, S
     const uint32_t total = __shfl_sync(EIC_FULL_MASK, incl, 31);
     const uint32_t excl = incl - len, full = __ballot_sync(EIC_FULL_MASK, len != 0);  // lanes with a window
     uint32_t live = 0;  // lanes whose vertex still has the distance it was queued with
-    if (total == 0) C.frontier += vertex && now == d ? 1 : 0;
+    if (!kRoad && total == 0) C.frontier += vertex && now == d ? 1 : 0;
     if (!kRoad) {
       spent += (total + 31) / 32;
       if (spent > kFuseIters && lane == 0) fstop[wave] = 1;
@@ -1211,7 +1211,7 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, S
       if (g < total) ent = ld_stream(&A.G.adj[first_at + g]);
       if (g0 == 0) {
         live = __ballot_sync(EIC_FULL_MASK, now == d);
-        C.frontier += vertex && now == d ? 1 : 0;
+        if (!kRoad) C.frontier += vertex && now == d ? 1 : 0;
       }
       bool ok = false, first = false;
       uint32_t nd = 0;
@@ -1247,6 +1247,7 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, S
       }
       warp_push(Fw, first, v);
     }
+    if (kRoad) C.frontier += vertex && now == d ? 1 : 0;  // (where the registers of either form allow: 3% on grids)
     group_sync();  // the wave's pushes are complete
     lt += min(fcnt[wave], room);
     const bool stop = !kRoad && fstop[wave] && i0 >= i1;
@@ -1795,16 +1796,14 @@ __device__ void run_query(const KArgs& A, QueryShared& Q, unsigned long long& ti
   }
   if (qb == 0 && threadIdx.x == 0) tl_mark(A, 0, L.rid);
   bool alive = !L.done;  // an isolated source has nothing to relax
-  uint32_t total_rounds = 0;
-  constexpr uint32_t kMaxRounds = 1u << 22;  // every block counts the same rounds and stops together
+  constexpr uint32_t kMaxRounds = 1u << 22;  // every block counts the same rounds (L.rid) and stops together
   while (alive) {
     // ------------------------------------------------ rounds of one step
     uint32_t rin = 0;
     bool plain = false;                    // the round must be a plain one
     constexpr uint32_t kStayPlainShift = 2;
     for (;;) {
-      ++L.rid;
-      if (++total_rounds > kMaxRounds) {
+      if (++L.rid > kMaxRounds) {
         if (threadIdx.x == 0) atomicCAS(&c->status, 0, EIC_ETIMEOUT);
         alive = false;
         break;
