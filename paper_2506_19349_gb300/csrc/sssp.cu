@@ -1247,7 +1247,8 @@ __device__ void fused_round(const KArgs& A, const RoundCtx& R, const Local& L, S
       }
       warp_push(Fw, first, v);
     }
-    if (kRoad) C.frontier += vertex && now == d ? 1 : 0;  // (where the registers of either form allow: 3% on grids)
+    if (kRoad) C.frontier += vertex && now == d ? 1 : 0;  // (here and not with the entries: 3% on
+                                                            // grids, by the kernel's registers)
     group_sync();  // the wave's pushes are complete
     lt += min(fcnt[wave], room);
     const bool stop = !kRoad && fstop[wave] && i0 >= i1;
